@@ -669,9 +669,8 @@ struct PairUnit {
 // Tiles of one claim unit of the dynamic weight-gradient schedule, from the expert's
 // k-blocks per tile: light experts' tiles (one to seven 128-row k-blocks) are claimed,
 // published to the pair and handed to the epilogue warps several at a time, about eight
-// k-blocks of work per claim. Each hand-off costs the single producer and MMA-issuer
-// threads ~2,000 cycles (a cluster-scope release and arrive), which one tile of one
-// k-block (~1,000 cycles of MMA) could not hide.
+// k-blocks of work per claim, so that a claim's global atomic is in flight behind enough
+// MMA work (one tile of one k-block has ~1,000 cycles of it).
 __host__ __device__ constexpr int unit_tiles(int nkb) {
   return nkb >= 8 ? 1 : nkb >= 4 ? 2 : nkb >= 2 ? 4 : 8;
 }
@@ -883,6 +882,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   // cost the same (and with p.dynamic == 0 the weight gradients' too): a unit is one tile,
   // and every role of a pair computes its unit numbers itself, cluster, cluster +
   // nclusters, ..., with no hand-off.
+  // The values reach the odd CTA by asynchronous stores counted on its barriers, and the
+  // epilogue warps give an accumulator back with a plain arrive: as cluster-scope releases
+  // these made each claim cost the producer ~3,300 cycles (they wait for the atomic and the
+  // loads in flight) and each tile of a warp ~1,900 cycles (its stores). Light experts' tiles
+  // ran at the epilogue's pace, ~5,600 cycles each, half of it that wait; without it ~3,900:
+  // dW_gate_up 214 -> 148 us at 698 tokens over 105 experts (d 2304, d_ff 768, top-6),
+  // 256 -> 188 us at 2,039 tokens over 64 (d 2048, d_ff 1408), 20.3 -> 19.6 ms at T=65536.
   auto static_unit = [&](uint32_t n) -> int {
     const int unit = cluster + int(n) * nclusters;
     return unit < total ? unit : -1;
@@ -897,12 +903,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (leader) {
       const int v = claimed < total ? claimed : -1;
       s_ring[slot] = v;
-      tc::st_cluster_u32(ring_peer + 4u * slot, v);
       tc::mbar_arrive(ring_bar(slot));
-      tc::mbar_arrive_cluster(ring_bar_peer + 8u * slot);
+      tc::st_async_u32(ring_peer + 4u * slot, v, ring_bar_peer + 8u * slot);
       if (v >= 0) claimed = nclusters + atomicAdd(p.sched_ctr, 1);
       return v;
     }
+    tc::mbar_arrive_expect_tx(ring_bar(slot), 4);  // the even CTA's asynchronous store
     if (!tc::mbar_wait_cluster(ring_bar(slot), (n / kRing) & 1u, kWaitLimitNs, abort_flag)) {
       fail(abort_flag);
       return -2;
@@ -1070,9 +1076,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           // the epilogue warps of both CTAs learn the unit (-1: no more units)
           const uint32_t e_slot = n & 1u;
           s_epi[e_slot] = unit;
-          tc::st_cluster_u32(epi_peer + 4u * e_slot, unit);
           tc::mbar_arrive(epi_bar(e_slot));
-          tc::mbar_arrive_cluster(epi_bar_peer + 8u * e_slot);
+          tc::st_async_u32(epi_peer + 4u * e_slot, unit, epi_bar_peer + 8u * e_slot);
         }
         if (unit < 0) break;
         tc::fence_after_sync();
@@ -1146,6 +1151,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int unit;
       if (dyn) {
         const uint32_t e_slot = n & 1u;
+        if (!leader && warp == 2 && lane == 0) tc::mbar_arrive_expect_tx(epi_bar(e_slot), 4);
         ok = tc::mbar_wait_cluster(epi_bar(e_slot), (n >> 1) & 1u, kWaitLimitNs, abort_flag);
         __syncwarp();
         if (!ok) { fail(abort_flag); break; }
@@ -1179,7 +1185,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           tc::fence_before_sync();
           __syncwarp();
-          if (lane == 0) tc::mbar_arrive_cluster(tempty_leader + 8u * a);
+          if (lane == 0) tc::mbar_arrive_remote(tempty_leader + 8u * a);
           if (mine) {
             const int trow = t.e * (p.m_tiles_w * BM) + mt * BM + q * 32;
 #pragma unroll
@@ -1198,7 +1204,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         tc::fence_before_sync();
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive_cluster(tempty_leader + 8u * a);
+        if (lane == 0) tc::mbar_arrive_remote(tempty_leader + 8u * a);
       }
     }
     if (lane == 0) tc::bulk_wait0();  // this warp's output stores are complete
