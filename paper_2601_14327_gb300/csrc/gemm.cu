@@ -99,6 +99,7 @@ struct GemmParams {
   const int32_t *group_offsets;  // [E+1], padded group starts (device)
   int E, d, F;
   int n_tiles;     // output column tiles
+  int n_cols;      // output columns; the last tile may be cut (a multiple of 128, see tile_cols)
   int m_tiles_w;   // weight-gradient modes: row tiles of one expert's output
   int nkb;         // k-blocks per tile (activation modes)
   uint16_t *out;   // primary output
@@ -244,6 +245,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams &p, const CUtenso
     float gsum = 0.f;  // this row's sum of dH * H over the warp's columns
 #pragma unroll 1
     for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
+      if (f0 + c >= F) break;  // a cut last tile
       uint4 va[4], vb[4];
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
@@ -296,6 +298,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams &p, const CUtenso
     if (router) dz = p.row_dz[row];
 #pragma unroll 1
     for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
+      if (nt * BN + c >= p.n_cols) break;  // a cut last tile
       uint32_t r[32];
       float w = 0.f;
       if (router) w = __ldg(p.w_router + size_t(nt * BN + c + lane) * p.E + e);
@@ -336,8 +339,8 @@ __device__ __forceinline__ void zero_fill_stage(uint32_t stage, int lane) {
 // half of output tile (trow, nt), as one bulk group.
 template <int BN>
 __device__ __forceinline__ void store_chunks_from(const CUtensorMap *tmO, uint32_t stage, int trow,
-                                                  int nt, int half) {
-  for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32)
+                                                  int nt, int half, int n_cols) {
+  for (int c = half * (BN / 2); c < (half + 1) * (BN / 2) && nt * BN + c < n_cols; c += 32)
     tc::tma_store_2d(tmO, stage, nt * BN + c, trow);
   tc::bulk_commit();
 }
@@ -345,7 +348,7 @@ __device__ __forceinline__ void store_chunks_from(const CUtensorMap *tmO, uint32
 // Zero weight gradient of an expert without rows: this warp's 32 rows and column half.
 template <int BN>
 __device__ __forceinline__ void zero_tile_store(const CUtensorMap *tmO, uint32_t stage, int lane,
-                                                int trow, int nt, int half) {
+                                                int trow, int nt, int half, int n_cols) {
   if (lane == 0) tc::bulk_wait_read0();
   __syncwarp();
   const uint4 z = make_uint4(0, 0, 0, 0);
@@ -354,7 +357,7 @@ __device__ __forceinline__ void zero_tile_store(const CUtensorMap *tmO, uint32_t
   tc::fence_proxy_async_smem();
   __syncwarp();
   if (lane == 0) {
-    for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32)
+    for (int c = half * (BN / 2); c < (half + 1) * (BN / 2) && nt * BN + c < n_cols; c += 32)
       tc::tma_store_2d(tmO, stage, nt * BN + c, trow);
     tc::bulk_commit();
   }
@@ -504,7 +507,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc::tma_load_2d(a_dst, &tmA, fb, k0, row0);
 #pragma unroll
             for (int i = 0; i < BN / 128; ++i)
-              tc::tma_load_2d(b_dst + i * 128 * 128, &tmB, fb, k0, t.e * p.d + t.nt * BN + i * 128);
+              tc::tma_load_2d(b_dst + i * 128 * 128, &tmB, fb, k0,
+                              t.nt * BN + i * 128 < p.n_cols ? t.e * p.d + t.nt * BN + i * 128 : -2 * BM);
           } else if (MODE == kDgradDown || MODE == kDgradGateUp) {
             const int row0 = t.goff + t.mt * BM;
             tc::tma_load_2d(a_dst, &tmA, fb, k0, row0);
@@ -582,7 +586,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (Tr::WGRAD && t.nkb == 0) {
         // empty group: its weight gradient is exactly zero
         const int M_out = p.m_tiles_w * BM;
-        zero_tile_store<BN>(&tmO, stage, lane, t.e * M_out + t.mt * BM + q * 32, t.nt, half);
+        zero_tile_store<BN>(&tmO, stage, lane, t.e * M_out + t.mt * BM + q * 32, t.nt, half, p.n_cols);
         continue;
       }
       const uint32_t a = tcount & 1u, aph = (tcount >> 1) & 1u;
@@ -1028,9 +1032,12 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int i = 0; i < BNH / 64; ++i)
                 tc::tma_load_2d_pair(b_dst + i * (KB * 128), &tmB, fb, t.nt * BN + int(rank) * BNH + i * 64, krow);
             } else {
-              // kGateUp: even CTA gate rows, odd CTA up rows; kDown: rows of W_down
-              const int brow = MODE == kGateUp ? t.e * 2 * p.F + int(rank) * p.F + t.nt * 128
-                                               : t.e * p.d + t.nt * BN + int(rank) * BNH;
+              // kGateUp: even CTA gate rows, odd CTA up rows; kDown: rows of W_down (zeros
+              // past the expert's last one)
+              const int bcol = t.nt * BN + int(rank) * BNH;
+              const int brow = MODE == kGateUp    ? t.e * 2 * p.F + int(rank) * p.F + t.nt * 128
+                               : bcol < p.n_cols ? t.e * p.d + bcol
+                                                 : -2 * BM;
 #pragma unroll
               for (int h = 0; h < KB / 64; ++h)
                 tc::tma_load_2d_pair(b_dst + h * (BNH * 128), &tmB, fb, k0 + h * 64, brow);
@@ -1141,7 +1148,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int e = s_order[E - n_pruned - n_empty + u / per_e];
           const int rem = u % per_e;
           const int mb = rem / p.n_tiles, nt = rem - mb * p.n_tiles;
-          if (lane == 0) store_chunks_from<BN>(&tmO, stage, e * M_out + mb * BM + q * 32, nt, half);
+          if (lane == 0) store_chunks_from<BN>(&tmO, stage, e * M_out + mb * BM + q * 32, nt, half, p.n_cols);
         }
       }
     }
@@ -1192,7 +1199,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int c = 0; c < BN / 2; c += 32) {
               uint4 v[4];
               pack32(*reinterpret_cast<const uint32_t(*)[32]>(&r[c]), v);
-              stage_and_store(&tmO, stage, lane, v, t.nt * BN + half * (BN / 2) + c, trow);
+              const int col = t.nt * BN + half * (BN / 2) + c;
+              if (col < p.n_cols) stage_and_store(&tmO, stage, lane, v, col, trow);
             }
           }
           continue;
@@ -1332,6 +1340,31 @@ bool split_rows(uint64_t rows) {
   return on && rows >= (uint64_t(1) << 18);
 }
 
+// Columns of an output tile, 256 or 128, for a tile list of about row_pairs (256-row pairs) x
+// column tiles. N is a multiple of 128; when it is not one of 256 the last 256-wide tile's
+// second half lies past the matrix: its operand boxes are zero-filled without memory reads and
+// it is not stored.
+// - Enough tiles: 256. A CTA of a 256-wide pair tile loads 64 KB per 128-deep k-block where a
+//   128-wide one loads 48 KB for half the columns, and at ~45 B per clock and SM those loads set
+//   the pace. 128-wide / 256-wide with a cut last tile: dH 140 / 122 us and dW_down 112 / 104 us
+//   at 2,039 tokens, top-6, 64 experts, d 2048, d_ff 1408; dX 1951 / 1593 us and dW_gate_up
+//   1970 / 1650 us at 65,396 tokens, top-6, 85 experts, d 2176, d_ff 768.
+// - A cut tile pays its unused half, so below three waves of tiles (the last wave weighs more
+//   then): 128. dH 13.9 / 20.0 us at 1,021 tokens, top-4, 32 experts, d 512, d_ff 384.
+// - Tiles of 256 for at most half the pairs: 128, twice as many pairs work for half as long.
+//   down 8.2 us against 9.1 us at 512 tokens, top-2, 16 experts, d 256, d_ff 512.
+int tile_cols(int N, int64_t row_pairs) {
+  if (N < 256) return 128;
+  const int64_t pairs = moe::num_sms() / 2, wide = row_pairs * ((N + 255) / 256);
+  if (2 * wide <= pairs) return 128;
+  return N % 256 == 0 || wide >= 3 * pairs ? 256 : 128;
+}
+// Row pairs of the activation GEMMs' tile lists, about: every expert's rows in pairs of
+// 128-row blocks, from the rows allocated (T*k + 128 E); half a pair more per expert.
+int64_t act_row_pairs(int64_t rows_cap, int E) {
+  return std::max<int64_t>(0, rows_cap - int64_t(128) * E) / 256 + (E + 1) / 2;
+}
+
 // Builds the tensor maps for one GEMM and launches it. A: [a_rows, a_cols] row-major
 // bf16; B likewise. N = output columns (for kGateUp: 2F, in tiles of 128 gate + 128 up).
 // The output p.out is [o_rows, o_cols] row-major bf16.
@@ -1357,8 +1390,11 @@ int run_gemm_out(int N, const void *a_base, uint64_t a_rows, uint64_t a_cols, co
   using Tr = Traits<MODE>;
   const bool pair = use_pair<MODE>();
   if (!Tr::WGRAD) p.dynamic = 0;  // equal-cost tiles: fixed stride, no counter to reset
-  const int BN = (MODE == kGateUp || N % 256 == 0) ? 256 : 128;
-  p.n_tiles = (MODE == kGateUp) ? N / 256 : N / BN;
+  const int BN = MODE == kGateUp ? 256
+                                 : tile_cols(N, Tr::WGRAD ? int64_t(p.E) * ((p.m_tiles_w + 1) / 2)
+                                                          : act_row_pairs(int64_t(a_rows), p.E));
+  p.n_tiles = (N + BN - 1) / BN;
+  p.n_cols = N;
   const bool gather = p.token_of_row != nullptr;
   if (gather && MODE != kGateUp && MODE != kWgradGateUp)
     return moe::set_error(MOE_ERR_UNSUPPORTED, "%s: no gathered operand in this GEMM", what);
@@ -1713,6 +1749,7 @@ int moe_grouped_ffn_bwd_dgrad(const uint16_t *d_out_perm, const uint16_t *ab_sav
   if (!router && !gate && (topk_gate || row_of_assignment))
     return moe::set_error(MOE_ERR_ARG, "%s: routing arguments without a router term or d_gate_out", fn);
   int64_t Rr = 0;
+  int gate_stride = 0;
   moe::WsLayout L{};
   if (router || gate) {
     if (T < 0 || k < 1 || k > 8 || k > E) return moe::set_error(MOE_ERR_ARG, "%s: T=%d k=%d", fn, T, k);
@@ -1732,8 +1769,10 @@ int moe_grouped_ffn_bwd_dgrad(const uint16_t *d_out_perm, const uint16_t *ab_sav
   p.out = d_ab;
   p.aux = ab_saved;
   if (gate) {
+    const int cols = tile_cols(F, act_row_pairs(rows_cap, E));
+    gate_stride = 2 * ((F + cols - 1) / cols);  // column halves of the N tiles
     p.gate_partial = reinterpret_cast<float *>(static_cast<char *>(ws) + L.gate_partial);
-    p.gate_stride = 2 * (F / (F % 256 == 0 ? 256 : 128));  // column halves of the N tiles
+    p.gate_stride = gate_stride;
   }
   if ((st = run_gemm<kDgradDown>(F, d_out_perm, R, d, w_down, uint64_t(E) * d, F, R, 2 * F, p,
                                  s, "moe_grouped_ffn_bwd: dH GEMM")))
@@ -1743,7 +1782,7 @@ int moe_grouped_ffn_bwd_dgrad(const uint16_t *d_out_perm, const uint16_t *ab_sav
   if (gate && A > 0) {
     MOE_LAUNCH("gate_from_rows", s, gate_from_rows_kernel<<<grid_for(A), 256, 0, s>>>(
                                         reinterpret_cast<const float *>(static_cast<char *>(ws) + L.gate_partial),
-                                        2 * (F / (F % 256 == 0 ? 256 : 128)), topk_gate,
+                                        gate_stride, topk_gate,
                                         row_of_assignment, A, Rr, d_gate_out));
     if ((st = moe::launch_status("moe_grouped_ffn_bwd_dgrad: gate gradient"))) return st;
   }

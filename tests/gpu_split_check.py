@@ -17,7 +17,8 @@ import torch  # noqa: E402
 from gpu_helpers import case_inputs, run_gpu_layer  # noqa: E402
 
 # T, d, E, k, F, bias: T*k + 128*E >= 2^18 grouped rows; skewed loads, so that many groups
-# have an odd number of blocks, some only one; d = 384 gives N = 128 tiles in down and dX
+# have an odd number of blocks, some only one; d = 384 gives a cut last column tile in down
+# and dX, d_ff = 128 N = 128 tiles in dH
 SPLIT_CASES = [
     (32768, 256, 64, 8, 256, "zipf"),
     (32768, 384, 128, 8, 128, "loguniform"),

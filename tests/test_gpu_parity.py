@@ -280,6 +280,18 @@ def test_layer_fwd_bwd_against_oracle(T, d, E, k, F, bias, n_masked):
         assert (b.dw_router[:, e].cpu().numpy() == 0).all()
 
 
+@pytest.mark.parametrize("T,d,E,k,F,bias,n_masked", [
+    # >= 3 waves of 256-wide tiles with a cut last one: in every GEMM whose N is 384 or 640
+    (6000, 384, 64, 4, 640, "zipf", 5),
+    # the same with 1 of 2 column tiles cut, one-block groups and empty experts
+    (5000, 640, 128, 3, 384, "loguniform", 0),
+    # 256-wide tiles would not fill half the CTA pairs: 128-wide ones, N a multiple of 256
+    (200, 256, 3, 2, 512, "none", 0),
+])
+def test_column_tile_widths_against_oracle(T, d, E, k, F, bias, n_masked):
+    test_layer_fwd_bwd_against_oracle(T, d, E, k, F, bias, n_masked)
+
+
 def test_tiny_workload_end_to_end_gpu_logits():
     """The tiny workload with the router computed on the GPU (no shared logits)."""
     T, d, E, k, F = 512, 256, 16, 2, 512
