@@ -78,7 +78,42 @@ int gemm_dev_error(int clear, int *code);
     nvtxRangePop();                                          \
   } while (0)
 
+namespace moe {
+// Launches a kernel as a programmatic dependent of the one before it on the stream: its
+// blocks may become resident, and run up to their pdl_wait(), while that kernel's last
+// blocks finish. EVERY kernel launched this way calls pdl_wait() in all its threads before it
+// touches memory, so stream order holds for every access, across any number of launches.
+// Without it a kernel started ~2 us after its predecessor's end (launch latency and drain),
+// and a layer is a dozen or two launches: with it and fewer launches a forward at T=512,
+// d=256, 16 experts takes 48 us instead of 69, a training step at T=1,021, d=512 140 instead of
+// 209.
+template <typename... P, typename... A>
+void launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, P(args)...);  // its error is read by launch_status()
+}
+}  // namespace moe
+
 // -------------------------------------------------------------- device side
+// Programmatic dependent launch (see launch_dep): waits until every kernel before this one
+// has completed and its writes are visible / lets the next kernel's blocks become resident.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_start() {
+  pdl_launch();
+  pdl_wait();
+}
 #define MOE_DEV_ERR_DECL static __device__ int g_dev_err;
 #define MOE_DEV_ERR_DEFINE_READER(fn)                                               \
   int fn(int clear, int *code) {                                                    \

@@ -126,10 +126,13 @@ struct GemmParams {
   // row's sum over its partials is g * <dy, O> (dH = g * dy W_down).
   float *gate_partial;
   int gate_stride;
+  // kDgradDown ahead of a dX GEMM with the router's term (nullptr: without): zeroed for every
+  // grouped row; the rows of assignments are written between the two GEMMs.
+  float *zero_dz;
   // Weight-gradient modes: experts with active_mask[e] == 0 (pruned by LAEP) get no tile
   // and no store; their gradient buffers are left as they are (nullptr: all experts live).
   const uint8_t *active_mask;
-  // CTA-pair kernel: tile counter of the dynamic schedule (zero at launch, 4 bytes of the
+  // CTA-pair kernel: tile counter of the dynamic schedule (zeroed before the launch, in the
   // caller's workspace); dynamic = 0 walks the list with a fixed stride instead.
   int *sched_ctr;
   int dynamic;
@@ -275,6 +278,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams &p, const CUtenso
       stage_and_store(tmO, stage, lane, vda, f0 + c, trow);
       stage_and_store(tmO, stage, lane, vdb, F + f0 + c, trow);
     }
+    if (p.zero_dz != nullptr && nt == 0 && half == 0) p.zero_dz[row] = 0.f;
     if (p.gate_partial != nullptr) p.gate_partial[row * p.gate_stride + nt * 2 + half] = gsum;
   } else {
     int trow;
@@ -422,6 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::tmem_alloc(tc::smem_u32(misc), Sh::TMEM_COLS);
     tc::tmem_relinquish();
   }
+  pdl_wait();  // barriers and TMEM are set up while the previous kernel ends
   // ---- tile schedule, built from the device-resident group offsets ----
   // Weight gradients: experts heaviest first (ties to the lower id), pruned experts
   // (active_mask 0) last with no tile, live experts without rows with tiles of zero
@@ -459,6 +464,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc::fence_after_sync();
   const uint32_t tmem_base = static_cast<uint32_t>(misc[0]);
   const int total = s_prefix[E];
+  pdl_launch();  // only now: a dependent must not take the TMEM columns this kernel waits for
 
   auto decode = [&](int tile) {
     int lo = 0, hi = E - 1;
@@ -764,6 +770,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::tmem_alloc_pair(tc::smem_u32(misc), Sh::TMEM_COLS);
     tc::tmem_relinquish_pair();
   }
+  pdl_wait();  // barriers and TMEM are set up while the previous kernel ends
   // ---- tile list: identical in both CTAs of every pair ----
   // Weight gradients (a tile costs as much as its expert has rows): experts in descending
   // order of rows (ties to the lower id), the longest-processing-time order of Algorithm
@@ -821,6 +828,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc::fence_after_sync();
   const uint32_t tmem_base = static_cast<uint32_t>(misc[0]);
   const int total = s_prefix[E];
+  pdl_launch();  // only now: a dependent must not take the TMEM columns this kernel waits for
 
   // Every role of a pair sees the pair's tiles in increasing order (a fixed stride, or
   // claims from a counter that only grows), so the expert of the next tile is found by
@@ -1254,6 +1262,19 @@ bool sched_dynamic() {
   return v == 1;
 }
 
+// The tile counters of the two weight-gradient launches of a call (first 8 bytes of the
+// caller's workspace) start at zero: one small launch for both (a memset node before each
+// GEMM cost ~1 us and two gaps, and kept the GEMM's set-up from overlapping its predecessor).
+__global__ void zero_sched_kernel(int *ctr) {
+  pdl_start();
+  if (threadIdx.x < 2) ctr[threadIdx.x] = 0;
+}
+int zero_sched(const GemmParams &p, cudaStream_t s, const char *what) {
+  if (!p.dynamic) return MOE_OK;
+  MOE_LAUNCH("zero_sched", s, moe::launch_dep(zero_sched_kernel, 1, 32, 0, s, p.sched_ctr));
+  return moe::launch_status(what);
+}
+
 // Points p at the tile counter in the first bytes of the caller's workspace.
 int use_sched_ws(GemmParams &p, void *ws, size_t ws_bytes, const char *fn) {
   if (!ws || !moe::aligned16(ws) || ws_bytes < moe::kGemmSchedBytes)
@@ -1276,7 +1297,8 @@ int launch_one(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o,
     if (e != cudaSuccess) return moe::cuda_status(e, what);
     attr = true;
   }
-  MOE_LAUNCH(kGemmName[MODE], s, grouped_gemm_kernel<MODE, BN><<<moe::num_sms(), kThreads, Sh::SMEM, s>>>(a, b, o, p));
+  MOE_LAUNCH(kGemmName[MODE], s, moe::launch_dep(grouped_gemm_kernel<MODE, BN>, moe::num_sms(), kThreads, Sh::SMEM, s,
+                                                 a, b, o, p));
   return moe::launch_status(what);
 }
 
@@ -1285,7 +1307,7 @@ int launch_pair(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o
                 const GemmParams &p, cudaStream_t s, const char *what) {
   using Sh = PairShape<BN, GATHER ? 64 : 128>;
   auto kern = grouped_gemm_pair_kernel<MODE, BN, GATHER>;
-  cudaLaunchAttribute at[2];
+  cudaLaunchAttribute at[3];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;
@@ -1299,6 +1321,8 @@ int launch_pair(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o
   }();
   at[1].id = cudaLaunchAttributePriority;
   at[1].val.priority = prio;
+  at[2].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see moe::launch_dep
+  at[2].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = Sh::SMEM;
@@ -1317,11 +1341,7 @@ int launch_pair(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o
     nclusters = n;
   }
   cfg.gridDim = dim3(2 * nclusters);
-  cfg.numAttrs = 2;
-  if (p.dynamic) {  // the tile counter starts at zero for every launch
-    cudaError_t e = cudaMemsetAsync(p.sched_ctr, 0, sizeof(int), s);
-    if (e != cudaSuccess) return moe::cuda_status(e, what);
-  }
+  cfg.numAttrs = 3;
   MOE_LAUNCH(kGemmName[MODE], s, cudaLaunchKernelEx(&cfg, kern, a, b, o, p));
   return moe::launch_status(what);
 }
@@ -1475,6 +1495,7 @@ __global__ void wait_timeout_selftest_kernel(uint64_t limit_ns) {
 // ---- combine in the down GEMM's epilogue: helpers ----
 // row_token[r] = -1 for every grouped row (padding rows keep it).
 __global__ void combine_rows_fill_kernel(int32_t *__restrict__ row_token, int64_t R) {
+  pdl_start();
   for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < R;
        r += int64_t(gridDim.x) * blockDim.x)
     row_token[r] = -1;
@@ -1484,6 +1505,7 @@ __global__ void combine_rows_scatter_kernel(const int32_t *__restrict__ row_of_a
                                             const float *__restrict__ topk_gate, int64_t A, int k,
                                             int64_t R, int32_t *__restrict__ row_token,
                                             float *__restrict__ row_gate) {
+  pdl_start();
   for (int64_t a = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; a < A;
        a += int64_t(gridDim.x) * blockDim.x) {
     const int32_t r = row_of_assignment[a];
@@ -1495,57 +1517,67 @@ __global__ void combine_rows_scatter_kernel(const int32_t *__restrict__ row_of_a
     }
   }
 }
-// The router's logit gradient of every assignment (softmax over the k selected experts:
-// dz_j = g_j (dg_j - sum_i g_i dg_i), summed in slot order with fused multiply-adds, as
-// moe_route_bwd computes it) written to the assignment's grouped row. Padding rows keep
-// the zeros the caller wrote first.
-__global__ void router_row_dz_kernel(const float *__restrict__ topk_gate,
-                                     const float *__restrict__ d_gate,
-                                     const int32_t *__restrict__ row_of_assignment, int T, int k,
-                                     int64_t R, float *__restrict__ row_dz) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x) {
-    float g[8], dg[8], s = 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      g[j] = 0.f;
-      dg[j] = 0.f;
-      if (j < k) {
-        g[j] = topk_gate[size_t(t) * k + j];
-        dg[j] = d_gate[size_t(t) * k + j];
-        s = fmaf(g[j], dg[j], s);
+// Between the dH and the dX GEMM, eight lanes per token (lane j = its slot j). GATE: d_gate[t, j]
+// = <dy[t], O[row(t, j)]> from the dH GEMM's per-row partial sums of dH * H (summed in a fixed
+// order), which equal g[t, j] * <dy[t], O[row]>; divided by the gate (positive for every
+// selected expert; 0 is written for a zero gate). ROUTER: the router's logit gradient of every
+// assignment (softmax over the k selected experts: dz_j = g_j (dg_j - sum_i g_i dg_i), summed in
+// slot order with fused multiply-adds, as moe_route_bwd computes it) at the assignment's grouped
+// row; padding rows keep the zeros that the dH GEMM's epilogue wrote. One launch for what were
+// two and a memset (2.9 + 1.7 + 2.5 us and three gaps at T=1,021, top-4).
+template <bool GATE, bool ROUTER>
+__global__ void row_gates_kernel(const float *__restrict__ partial, int stride,
+                                 const float *__restrict__ topk_gate,
+                                 const int32_t *__restrict__ row_of_assignment, int T, int k, int64_t R,
+                                 const float *__restrict__ d_gate_in, float *__restrict__ d_gate_out,
+                                 float *__restrict__ row_dz) {
+  pdl_start();
+  const int j = threadIdx.x & 7;
+  const int64_t n = (int64_t(T) * 8 + 31) & ~int64_t(31);  // whole warps
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n;
+       i += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t t = i >> 3, a = t * k + j;
+    float g = 0.f, dg = 0.f;
+    int r = -1;
+    const bool mine = t < T && j < k;
+    if (mine) {
+      g = topk_gate[a];
+      r = row_of_assignment[a];
+      const bool ok = r >= 0 && r < R;
+      if (!ok) {
+        dev_flag(&g_dev_err, MOE_DEV_ROWS_OVERFLOW);
+        r = -1;
+      }
+      if (GATE) {
+        if (ok) {
+          float s = 0.f;
+          const float2 *src = reinterpret_cast<const float2 *>(partial + size_t(r) * stride);
+#pragma unroll 4
+          for (int c = 0; c < stride / 2; ++c) {
+            const float2 v = src[c];
+            s += v.x;
+            s += v.y;
+          }
+          dg = g > 0.f ? s / g : 0.f;
+          d_gate_out[a] = dg;
+        }
+      } else {
+        dg = d_gate_in[a];
       }
     }
+    if (ROUTER) {
+      float s = 0.f;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (j < k) {
-        const int32_t r = row_of_assignment[size_t(t) * k + j];
-        if (r >= 0 && r < R) row_dz[r] = g[j] * (dg[j] - s);
-        else dev_flag(&g_dev_err, MOE_DEV_ROWS_OVERFLOW);
+      for (int q = 0; q < 8; ++q) {
+        const float gq = __shfl_sync(0xffffffffu, g, q, 8), dgq = __shfl_sync(0xffffffffu, dg, q, 8);
+        if (q < k) s = fmaf(gq, dgq, s);
       }
+      if (mine && r >= 0) row_dz[r] = g * (dg - s);
     }
-  }
-}
-// d_gate[t, j] = <dy[t], O[row(t, j)]> from the dH GEMM's per-row partial sums of dH * H
-// (summed in a fixed order), which equal g[t, j] * <dy[t], O[row]>; divided by the gate
-// (positive for every selected expert; 0 is written for a zero gate).
-__global__ void gate_from_rows_kernel(const float *__restrict__ partial, int stride,
-                                      const float *__restrict__ topk_gate,
-                                      const int32_t *__restrict__ row_of_assignment, int64_t A,
-                                      int64_t R, float *__restrict__ d_gate) {
-  for (int64_t a = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; a < A;
-       a += int64_t(gridDim.x) * blockDim.x) {
-    const int32_t r = row_of_assignment[a];
-    if (r < 0 || r >= R) {
-      dev_flag(&g_dev_err, MOE_DEV_ROWS_OVERFLOW);
-      continue;
-    }
-    float s = 0.f;
-    for (int i = 0; i < stride; ++i) s += partial[size_t(r) * stride + i];
-    const float g = topk_gate[a];
-    d_gate[a] = g > 0.f ? s / g : 0.f;
   }
 }
 __global__ void zero_f32x4_kernel(float4 *__restrict__ p, int64_t n4) {
+  pdl_start();
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n4;
        i += int64_t(gridDim.x) * blockDim.x)
     p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1553,6 +1585,7 @@ __global__ void zero_f32x4_kernel(float4 *__restrict__ p, int64_t n4) {
 // y = bf16(y_acc), 8 elements per thread (n8 = T*d/8).
 __global__ void f32_to_bf16_kernel(const float4 *__restrict__ src, uint4 *__restrict__ dst,
                                    int64_t n8) {
+  pdl_start();
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n8;
        i += int64_t(gridDim.x) * blockDim.x) {
     const float4 a = src[2 * i], b = src[2 * i + 1];
@@ -1650,13 +1683,11 @@ int moe_grouped_ffn_fwd_combine(const uint16_t *x_perm, const int32_t *group_off
     return st;
   const int64_t A = int64_t(T) * k, n = int64_t(T) * d;
   if (T > 0) {
-    MOE_LAUNCH("combine_rows_fill", s, combine_rows_fill_kernel<<<grid_for(Rr), 256, 0, s>>>(row_token, Rr));
+    MOE_LAUNCH("combine_rows_fill", s, moe::launch_dep(combine_rows_fill_kernel, grid_for(Rr), 256, 0, s, row_token, Rr));
     if (int st = moe::launch_status("moe_grouped_ffn_fwd_combine: row fill")) return st;
-    MOE_LAUNCH("combine_rows_scatter", s, combine_rows_scatter_kernel<<<grid_for(A), 256, 0, s>>>(
-                                              row_of_assignment, topk_gate, A, k, Rr, row_token, row_gate));
+    MOE_LAUNCH("combine_rows_scatter", s, moe::launch_dep(combine_rows_scatter_kernel, grid_for(A), 256, 0, s, row_of_assignment, topk_gate, A, k, Rr, row_token, row_gate));
     if (int st = moe::launch_status("moe_grouped_ffn_fwd_combine: row scatter")) return st;
-    MOE_LAUNCH("zero_y_acc", s, zero_f32x4_kernel<<<grid_for(n / 4), 256, 0, s>>>(
-                                    reinterpret_cast<float4 *>(y_acc), n / 4));
+    MOE_LAUNCH("zero_y_acc", s, moe::launch_dep(zero_f32x4_kernel, grid_for(n / 4), 256, 0, s, reinterpret_cast<float4 *>(y_acc), n / 4));
     if (int st = moe::launch_status("moe_grouped_ffn_fwd_combine: zero")) return st;
   }
   // O = H W_down^T, combined into y_acc by the epilogue (O itself stored only if asked)
@@ -1678,8 +1709,7 @@ int moe_grouped_ffn_fwd_combine(const uint16_t *x_perm, const int32_t *group_off
                                    "moe_grouped_ffn_fwd_combine: down GEMM"))
     return st;
   if (T == 0) return MOE_OK;
-  MOE_LAUNCH("combine_y_bf16", s, f32_to_bf16_kernel<<<grid_for(n / 8), 256, 0, s>>>(
-                                      reinterpret_cast<const float4 *>(y_acc), reinterpret_cast<uint4 *>(y), n / 8));
+  MOE_LAUNCH("combine_y_bf16", s, moe::launch_dep(f32_to_bf16_kernel, grid_for(n / 8), 256, 0, s, reinterpret_cast<const float4 *>(y_acc), reinterpret_cast<uint4 *>(y), n / 8));
   return moe::launch_status("moe_grouped_ffn_fwd_combine: bf16 output");
 }
 
@@ -1774,28 +1804,28 @@ int moe_grouped_ffn_bwd_dgrad(const uint16_t *d_out_perm, const uint16_t *ab_sav
     p.gate_partial = reinterpret_cast<float *>(static_cast<char *>(ws) + L.gate_partial);
     p.gate_stride = gate_stride;
   }
+  float *row_dz = router ? reinterpret_cast<float *>(static_cast<char *>(ws) + L.row_dz) : nullptr;
+  p.zero_dz = row_dz;
   if ((st = run_gemm<kDgradDown>(F, d_out_perm, R, d, w_down, uint64_t(E) * d, F, R, 2 * F, p,
                                  s, "moe_grouped_ffn_bwd: dH GEMM")))
     return st;
-  p.gate_partial = nullptr;
-  const int64_t A = int64_t(T) * k;
-  if (gate && A > 0) {
-    MOE_LAUNCH("gate_from_rows", s, gate_from_rows_kernel<<<grid_for(A), 256, 0, s>>>(
-                                        reinterpret_cast<const float *>(static_cast<char *>(ws) + L.gate_partial),
-                                        gate_stride, topk_gate,
-                                        row_of_assignment, A, Rr, d_gate_out));
-    if ((st = moe::launch_status("moe_grouped_ffn_bwd_dgrad: gate gradient"))) return st;
+  if (T > 0 && (gate || router)) {
+    const float *part = p.gate_partial;
+    const int stride = p.gate_stride, grid = grid_for(int64_t(T) * 8);
+    if (gate && router)
+      MOE_LAUNCH("row_gates", s, moe::launch_dep(row_gates_kernel<true, true>, grid, 256, 0, s, part, stride, topk_gate,
+                                                 row_of_assignment, T, k, Rr, d_gate, d_gate_out, row_dz));
+    else if (gate)
+      MOE_LAUNCH("row_gates", s, moe::launch_dep(row_gates_kernel<true, false>, grid, 256, 0, s, part, stride, topk_gate,
+                                                 row_of_assignment, T, k, Rr, d_gate, d_gate_out, row_dz));
+    else
+      MOE_LAUNCH("row_gates", s, moe::launch_dep(row_gates_kernel<false, true>, grid, 256, 0, s, part, stride, topk_gate,
+                                                 row_of_assignment, T, k, Rr, d_gate, d_gate_out, row_dz));
+    if ((st = moe::launch_status("moe_grouped_ffn_bwd_dgrad: gate gradient and router rows"))) return st;
   }
+  p.zero_dz = nullptr;
+  p.gate_partial = nullptr;
   if (router) {
-    float *row_dz = reinterpret_cast<float *>(static_cast<char *>(ws) + L.row_dz);
-    cudaError_t e = cudaMemsetAsync(row_dz, 0, size_t(Rr) * 4, s);
-    if (e != cudaSuccess) return moe::cuda_status(e, "moe_grouped_ffn_bwd_dgrad: zero row_dz");
-    if (T > 0) {
-      MOE_LAUNCH("router_row_dz", s, router_row_dz_kernel<<<grid_for(T), 256, 0, s>>>(
-                                         topk_gate, gate ? d_gate_out : d_gate, row_of_assignment,
-                                         T, k, Rr, row_dz));
-      if ((st = moe::launch_status("moe_grouped_ffn_bwd_dgrad: router rows"))) return st;
-    }
     p.row_dz = row_dz;
     p.w_router = w_router;
   }
@@ -1824,6 +1854,7 @@ int moe_grouped_ffn_bwd_wgrad(const uint16_t *d_out_perm, const uint16_t *x_perm
   p.group_offsets = group_offsets;
   p.active_mask = active_mask;
   p.E = E; p.d = d; p.F = F;
+  if ((st = zero_sched(p, s, "moe_grouped_ffn_bwd: tile counters"))) return st;
   // dW_down[e] = dO_e^T H_e   ([d, F])
   p.nkb = 0;
   p.m_tiles_w = d / BM;
@@ -1832,6 +1863,7 @@ int moe_grouped_ffn_bwd_wgrad(const uint16_t *d_out_perm, const uint16_t *x_perm
                                  "moe_grouped_ffn_bwd: dW_down GEMM")))
     return st;
   // dW_gate_up[e] = [dA | dB]_e^T X_e   ([2F, d])
+  p.sched_ctr += 1;
   p.m_tiles_w = 2 * F / BM;
   p.out = dw_gate_up;
   return run_gemm<kWgradGateUp>(d, d_ab, R, 2 * F, x_perm, R, d, uint64_t(E) * 2 * F, d, p, s,
@@ -1860,12 +1892,14 @@ int moe_grouped_ffn_bwd_wgrad_gather(const uint16_t *d_out_perm, const uint16_t 
   p.group_offsets = group_offsets;
   p.active_mask = active_mask;
   p.E = E; p.d = d; p.F = F;
+  if ((st = zero_sched(p, s, "moe_grouped_ffn_bwd_wgrad_gather: tile counters"))) return st;
   p.nkb = 0;
   p.m_tiles_w = d / BM;
   p.out = dw_down;
   if ((st = run_gemm<kWgradDown>(F, d_out_perm, R, d, h, R, F, uint64_t(E) * d, F, p, s,
                                  "moe_grouped_ffn_bwd_wgrad_gather: dW_down GEMM")))
     return st;
+  p.sched_ctr += 1;
   p.m_tiles_w = 2 * F / BM;
   p.out = dw_gate_up;
   p.token_of_row = token_of_row;

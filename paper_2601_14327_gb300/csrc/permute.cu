@@ -5,6 +5,7 @@
 // deterministic and bit-exact. Groups start at multiples of 128 rows so that
 // every 128-row GEMM tile belongs to one expert; padding rows are zero.
 #include <cuda.h>
+#include <limits.h>
 
 #include <mutex>
 
@@ -17,119 +18,149 @@ namespace {
 constexpr int kChunk = moe::kPermChunk;  // assignments per block
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kPerWarp = kChunk / kWarps;  // 512 assignments per warp
+constexpr int kRankThreads = 1024;
+constexpr int kRankWarps = kRankThreads / 32;
+constexpr int kRankSteps = kChunk / kRankThreads;  // 32-wide steps of a warp
+constexpr int kRankGroups = kRankThreads / 256;    // threads per expert in the prefix
 
-// Block histograms: hist[e * nblk + b] = #{a in chunk b : idx[a] == e}.
-__global__ void __launch_bounds__(kThreads) perm_hist_kernel(const int32_t *__restrict__ idx,
-                                                             int64_t A, int E, int nblk,
-                                                             int32_t *__restrict__ hist) {
+// Block histograms: hist[b * E + e] = #{a in chunk b : idx[a] == e}.
+__global__ void __launch_bounds__(kRankThreads) perm_hist_kernel(const int32_t *__restrict__ idx,
+                                                                 int64_t A, int E,
+                                                                 int32_t *__restrict__ hist) {
   __shared__ int sh[256];
-  for (int e = threadIdx.x; e < E; e += kThreads) sh[e] = 0;
+  for (int e = threadIdx.x; e < E; e += kRankThreads) sh[e] = 0;
   __syncthreads();
+  pdl_start();
   const int64_t a0 = int64_t(blockIdx.x) * kChunk;
   const int64_t a1 = min(A, a0 + kChunk);
-  for (int64_t a = a0 + threadIdx.x; a < a1; a += kThreads) {
+  for (int64_t a = a0 + threadIdx.x; a < a1; a += kRankThreads) {
     const int e = idx[a];
     if (e >= 0 && e < E) atomicAdd(&sh[e], 1);
     else dev_flag(&g_dev_err, MOE_DEV_BAD_EXPERT);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < E; e += kThreads) hist[size_t(e) * nblk + blockIdx.x] = sh[e];
+  for (int e = threadIdx.x; e < E; e += kRankThreads) hist[size_t(blockIdx.x) * E + e] = sh[e];
 }
 
-// One CTA of 1024 threads: per-expert exclusive scan over blocks (in place),
-// group counts, and the padded group offsets.
-__global__ void __launch_bounds__(1024) perm_scan_kernel(
-    int32_t *__restrict__ hist, int E, int nblk, const int32_t *__restrict__ counts_check,
-    int64_t rows_cap, int32_t *__restrict__ group_offsets, int32_t *__restrict__ group_counts) {
-  __shared__ int s_cnt[256];
-  __shared__ int s_pad[257];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int e = warp; e < E; e += 32) {
-    int running = 0;
-    int32_t *h = hist + size_t(e) * nblk;
-    for (int base = 0; base < nblk; base += 32) {
-      const int v = (base + lane < nblk) ? h[base + lane] : 0;
-      int incl = v;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += o;
-      }
-      if (base + lane < nblk) h[base + lane] = running + incl - v;
-      running += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) s_cnt[e] = running;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int e = 0; e < E; ++e) {
-      s_pad[e] = acc;
-      acc += (s_cnt[e] + moe::kGroupPad - 1) / moe::kGroupPad * moe::kGroupPad;
-    }
-    s_pad[E] = acc;
-    if (int64_t(acc) > rows_cap) dev_flag(&g_dev_err, MOE_DEV_ROWS_OVERFLOW);
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e <= E; e += blockDim.x) group_offsets[e] = s_pad[e];
-  for (int e = threadIdx.x; e < E; e += blockDim.x) {
-    group_counts[e] = s_cnt[e];
-    if (counts_check != nullptr && counts_check[e] != s_cnt[e])
-      dev_flag(&g_dev_err, MOE_DEV_COUNT_MISMATCH);
-  }
-}
-
-// Row of every assignment: group start + rank among the earlier assignments
-// of the same expert. Warps walk consecutive sub-chunks in order; inside a
-// 32-wide step, lanes with equal experts are ranked by lane order.
-__global__ void __launch_bounds__(kThreads) perm_rank_kernel(
-    const int32_t *__restrict__ idx, int64_t A, int E, int nblk,
-    const int32_t *__restrict__ hist_prefix, const int32_t *__restrict__ group_offsets,
-    int64_t rows_cap, int32_t *__restrict__ row_of_assignment, int k,
+// Row of every assignment: group start + rank among the earlier assignments of the same
+// expert; group counts and padded group offsets (written by block 0). Latency-bound (a few
+// 16 KB chunks), so a block does in registers and shared memory what took three launches:
+// - ranks inside the block: warps own consecutive 128-assignment sub-chunks in 32-wide steps;
+//   lanes with equal experts are ranked by lane order, earlier steps by a per-warp count;
+// - the counts of the chunks before it and of all chunks, from the block histograms (one pass
+//   over nblk * E entries from L2 per block; a single chunk needs no histogram kernel);
+// - the scan of the padded group sizes (every block, 8 warps).
+// Histogram + scan + rank kernels took 5.7 + 4.5 + 8.4 us and two gaps at T=16384, top-8, 64
+// experts (32 chunks), 2.9 + 2.8 + 7.7 us at T=512, top-2; one kernel takes 5.2 us there now.
+__global__ void __launch_bounds__(kRankThreads) perm_rank_kernel(
+    const int32_t *__restrict__ idx, int64_t A, int E, int nblk, const int32_t *__restrict__ hist,
+    const int32_t *__restrict__ counts_check, int64_t rows_cap, int32_t *__restrict__ group_offsets,
+    int32_t *__restrict__ group_counts, int32_t *__restrict__ row_of_assignment, int k,
     int32_t *__restrict__ token_of_row) {
-  __shared__ int wh[kWarps][256];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < kWarps * 256; i += kThreads) (&wh[0][0])[i] = 0;
+  __shared__ int wh[kRankWarps][256];  // assignments of each warp to each expert, then their first row
+  __shared__ int part[kRankGroups][2][256];
+  __shared__ int s_warp[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < kRankWarps * 256; i += kRankThreads) (&wh[0][0])[i] = 0;
   __syncthreads();
-  const int64_t a0 = int64_t(blockIdx.x) * kChunk + int64_t(warp) * kPerWarp;
-  for (int s = 0; s < kPerWarp; s += 32) {
-    const int64_t a = a0 + s + lane;
-    if (a < A) {
-      const int e = idx[a];
-      if (e >= 0 && e < E) atomicAdd(&wh[warp][e], 1);
-    }
-  }
-  __syncthreads();
-  const bool overflow = group_offsets[E] > rows_cap;
-  for (int e = threadIdx.x; e < E; e += kThreads) {
-    int running = group_offsets[e] + hist_prefix[size_t(e) * nblk + blockIdx.x];
+  pdl_start();
+  const int64_t a0 = int64_t(blockIdx.x) * kChunk + int64_t(warp) * (kRankSteps * 32) + lane;
+  int e[kRankSteps], pos[kRankSteps];
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      const int c = wh[w][e];
-      wh[w][e] = running;
-      running += c;
+  for (int s = 0; s < kRankSteps; ++s) {
+    const int64_t a = a0 + s * 32;
+    e[s] = -1;
+    if (a < A) {
+      e[s] = idx[a];
+      if (e[s] < 0 || e[s] >= E) {
+        e[s] = -1;
+        dev_flag(&g_dev_err, MOE_DEV_BAD_EXPERT);
+      }
+    }
+  }
+  const int ex = tid & 255, grp = tid >> 8;
+  if (nblk > 1) {
+    int before = 0, all = 0;
+    if (ex < E) {
+#pragma unroll 8
+      for (int b = grp; b < nblk; b += kRankGroups) {
+        const int v = hist[size_t(b) * E + ex];
+        all += v;
+        if (b < int(blockIdx.x)) before += v;
+      }
+    }
+    part[grp][0][ex] = before;
+    part[grp][1][ex] = all;
+  }
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int s = 0; s < kRankSteps; ++s) {
+    const unsigned peers = __match_any_sync(0xffffffffu, e[s]);
+    pos[s] = __popc(peers & lt);
+    if (e[s] >= 0) pos[s] += wh[warp][e[s]];
+    __syncwarp();
+    if (e[s] >= 0 && lane == __ffs(peers) - 1) wh[warp][e[s]] += __popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+  // thread ex of the first 256: the expert's counts per warp -> exclusive, its total, its group
+  if (tid < 256) {
+    int own = 0;
+#pragma unroll 8
+    for (int w = 0; w < kRankWarps; ++w) {
+      const int c = wh[w][ex];
+      wh[w][ex] = own;
+      own += c;
+    }
+    int before = 0, cnt = own;
+    if (nblk > 1) {
+      cnt = 0;
+#pragma unroll
+      for (int g = 0; g < kRankGroups; ++g) {
+        before += part[g][0][ex];
+        cnt += part[g][1][ex];
+      }
+    }
+    if (ex >= E) cnt = 0;
+    const int padded = (cnt + moe::kGroupPad - 1) / moe::kGroupPad * moe::kGroupPad;
+    int incl = padded;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += v;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    int base = incl - padded, total = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      if (w < warp) base += s_warp[w];
+      total += s_warp[w];
+    }
+    const bool overflow = int64_t(total) > rows_cap;
+    part[0][0][ex] = overflow ? INT_MIN : base + before;  // first row of this block's assignments
+    if (blockIdx.x == 0) {
+      if (ex < E) {
+        group_offsets[ex] = base;
+        group_counts[ex] = cnt;
+        if (counts_check != nullptr && counts_check[ex] != cnt)
+          dev_flag(&g_dev_err, MOE_DEV_COUNT_MISMATCH);
+      }
+      if (tid == 0) {
+        group_offsets[E] = total;
+        if (overflow) dev_flag(&g_dev_err, MOE_DEV_ROWS_OVERFLOW);
+      }
     }
   }
   __syncthreads();
-  const unsigned lt = (1u << lane) - 1u;
-  for (int s = 0; s < kPerWarp; s += 32) {
-    const int64_t a = a0 + s + lane;
-    int e = -1;
-    if (a < A) {
-      e = idx[a];
-      if (e < 0 || e >= E) e = -1;
-    }
-    const unsigned peers = __match_any_sync(0xffffffffu, e);
-    const int rank = __popc(peers & lt);
-    const int leader = __ffs(peers) - 1;
+#pragma unroll
+  for (int s = 0; s < kRankSteps; ++s) {
+    const int64_t a = a0 + s * 32;
+    if (a >= A) continue;
     int row = -1;
-    if (e >= 0) row = wh[warp][e] + rank;
-    __syncwarp();
-    if (e >= 0 && lane == leader) wh[warp][e] += __popc(peers);
-    __syncwarp();
-    if (a < A) row_of_assignment[a] = (e >= 0 && !overflow) ? row : -1;
-    if (token_of_row != nullptr && a < A && e >= 0 && !overflow) token_of_row[row] = int(a / k);
+    if (e[s] >= 0 && part[0][0][e[s]] != INT_MIN) row = part[0][0][e[s]] + wh[warp][e[s]] + pos[s];
+    row_of_assignment[a] = row;
+    if (token_of_row != nullptr && row >= 0) token_of_row[row] = int(a / k);
   }
 }
 
@@ -139,17 +170,42 @@ __global__ void __launch_bounds__(kThreads) pad_token_kernel(const int32_t *__re
                                                              const int32_t *__restrict__ group_counts,
                                                              int E, int64_t rows_cap,
                                                              int32_t *__restrict__ token_of_row) {
+  pdl_start();
   const int e = blockIdx.x;
   const int r0 = group_offsets[e] + group_counts[e];
   const int r1 = int(min((long long)group_offsets[e + 1], (long long)rows_cap));
   for (int r = r0 + threadIdx.x; r < r1; r += kThreads) token_of_row[r] = 0;
 }
 
-// One warp per token: read x[t,:] once, write it to its k grouped rows.
+// Zeroes the padding rows [group_offsets[e] + group_counts[e], group_offsets[e+1]) of expert
+// b / kPadSplit, share b % kPadSplit. The first E * kPadSplit blocks of the kernels that
+// write a grouped tensor do this beside the token rows (as a launch of its own it took
+// 8 us of a 240 us dispatch at T=16384, d=4096, 64 experts, and 2-3 us of a small one).
+constexpr int kPadSplit = 8;
+__device__ __forceinline__ void zero_pad_rows(int b, const int32_t *__restrict__ group_offsets,
+                                              const int32_t *__restrict__ group_counts, int d,
+                                              int64_t rows_cap, uint16_t *__restrict__ buf) {
+  const int e = b / kPadSplit;
+  const int r0 = group_offsets[e] + group_counts[e];
+  const int r1 = int(min((long long)group_offsets[e + 1], (long long)rows_cap));
+  const int nv = d / 8;
+  const uint4 z = make_uint4(0, 0, 0, 0);
+  for (int r = r0 + (b % kPadSplit) * kWarps + int(threadIdx.x >> 5); r < r1; r += kPadSplit * kWarps)
+    for (int c = threadIdx.x & 31; c < nv; c += 32) stg_v4(buf + size_t(r) * d + c * 8, z);
+}
+
+// One warp per token: read x[t,:] once, write it to its k grouped rows. Blocks below
+// pad_blocks zero padding rows.
 __global__ void __launch_bounds__(kThreads) perm_gather_kernel(
     const uint16_t *__restrict__ x, const int32_t *__restrict__ row_of_assignment, int T, int d,
-    int k, int64_t rows_cap, uint16_t *__restrict__ x_perm) {
-  const int warp = (blockIdx.x * kThreads + threadIdx.x) >> 5;
+    int k, int64_t rows_cap, int pad_blocks, const int32_t *__restrict__ group_offsets,
+    const int32_t *__restrict__ group_counts, uint16_t *__restrict__ x_perm) {
+  pdl_start();
+  if (int(blockIdx.x) < pad_blocks) {
+    zero_pad_rows(blockIdx.x, group_offsets, group_counts, d, rows_cap, x_perm);
+    return;
+  }
+  const int warp = ((blockIdx.x - pad_blocks) * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= T) return;
   const int t = warp;
@@ -176,31 +232,11 @@ __global__ void __launch_bounds__(kThreads) perm_gather_kernel(
   }
 }
 
-// Zero the padding rows [group_offsets[e] + group_counts[e], group_offsets[e+1]);
-// blockIdx.x = expert, blockIdx.y splits that expert's padding rows.
-__global__ void __launch_bounds__(kThreads) pad_zero_kernel(const int32_t *__restrict__ group_offsets,
-                                                            const int32_t *__restrict__ group_counts,
-                                                            int E, int d, int64_t rows_cap,
-                                                            uint16_t *__restrict__ buf) {
-  const int e = blockIdx.x;
-  const int r0 = group_offsets[e] + group_counts[e];
-  const int r1 = int(min((long long)group_offsets[e + 1], (long long)rows_cap));
-  const int nv = d / 8;
-  const uint4 z = make_uint4(0, 0, 0, 0);
-  const int64_t n = int64_t(r1 - r0) * nv;
-  for (int64_t i = int64_t(blockIdx.y) * kThreads + threadIdx.x; i < n;
-       i += int64_t(gridDim.y) * kThreads) {
-    const int64_t r = r0 + i / nv, c = i % nv;
-    stg_v4(buf + size_t(r) * d + c * 8, z);
-  }
-}
-
-constexpr int kPadSplit = 8;  // blocks per expert in pad_zero_kernel
-
 // y[t] = sum_j g[t,j] * out_perm[row(t,j)]  (fp32 sum, one bf16 rounding)
 __global__ void __launch_bounds__(kThreads) combine_kernel(
     const uint16_t *__restrict__ out_perm, const int32_t *__restrict__ row_of_assignment,
     const float *__restrict__ gate, int T, int d, int k, uint16_t *__restrict__ y) {
+  pdl_start();
   const int warp = (blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= T) return;
@@ -237,13 +273,21 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(
 // d_out_perm[row(t,j)] = g[t,j] * dy[t];  d_gate[t,j] = <dy[t], out_perm[row(t,j)]>
 // DOUT: d_out_perm rows = g * dy[t]; DGATE: d_gate = <dy[t], out_perm rows>. The two
 // halves can run as separate launches (DGATE alone reads out_perm and writes nothing
-// large; DOUT alone never reads out_perm).
+// large; DOUT alone never reads out_perm). Blocks below pad_blocks (DOUT only) zero
+// padding rows of d_out_perm.
 template <bool DOUT, bool DGATE>
 __global__ void __launch_bounds__(kThreads) combine_bwd_kernel(
     const uint16_t *__restrict__ dy, const uint16_t *__restrict__ out_perm,
     const int32_t *__restrict__ row_of_assignment, const float *__restrict__ gate, int T, int d,
-    int k, int64_t rows_cap, uint16_t *__restrict__ d_out_perm, float *__restrict__ d_gate) {
-  const int warp = (blockIdx.x * kThreads + threadIdx.x) >> 5;
+    int k, int64_t rows_cap, int pad_blocks, const int32_t *__restrict__ group_offsets,
+    const int32_t *__restrict__ group_counts, uint16_t *__restrict__ d_out_perm,
+    float *__restrict__ d_gate) {
+  pdl_start();
+  if (DOUT && int(blockIdx.x) < pad_blocks) {
+    zero_pad_rows(blockIdx.x, group_offsets, group_counts, d, rows_cap, d_out_perm);
+    return;
+  }
+  const int warp = ((blockIdx.x - pad_blocks) * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= T) return;
   const int t = warp;
@@ -300,6 +344,7 @@ __global__ void __launch_bounds__(kThreads) combine_bwd_kernel(
 // w_t[e, i] = w[i, e]
 __global__ void transpose_router_kernel(const float *__restrict__ w, int d, int E,
                                         float *__restrict__ w_t) {
+  pdl_start();
   __shared__ float tile[32][33];
   const int i0 = blockIdx.x * 32, e0 = blockIdx.y * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -318,6 +363,7 @@ __global__ void __launch_bounds__(kThreads) permute_bwd_kernel(
     const uint16_t *__restrict__ dx_perm, const int32_t *__restrict__ row_of_assignment,
     const int32_t *__restrict__ topk_idx, const float *__restrict__ d_logits,
     const float *__restrict__ w_t, int T, int d, int E, int k, uint16_t *__restrict__ dx) {
+  pdl_start();
   const int warp = (blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= T) return;
@@ -370,6 +416,31 @@ __global__ void __launch_bounds__(kThreads) permute_bwd_kernel(
 
 int warp_grid(int T) { return (T + kWarps - 1) / kWarps; }
 
+// The grouped layout: group_offsets, group_counts, row_of_assignment (and token_of_row when
+// given). One chunk of assignments is one launch; more take the block histograms first.
+int launch_layout(const int32_t *idx, int64_t A, int E, int32_t *hist, const int32_t *counts,
+                  int64_t rows_cap, int32_t *group_offsets, int32_t *group_counts, int32_t *row, int k,
+                  int32_t *token_of_row, cudaStream_t s, const char *what) {
+  const int nblk = int(std::max<int64_t>(1, (A + kChunk - 1) / kChunk));
+  if (nblk > 1) {
+    MOE_LAUNCH("perm_hist", s, moe::launch_dep(perm_hist_kernel, nblk, kRankThreads, 0, s, idx, A, E, hist));
+    if (int st = moe::launch_status(what)) return st;
+  }
+  MOE_LAUNCH("perm_rank", s, moe::launch_dep(perm_rank_kernel, nblk, kRankThreads, 0, s, idx, A, E, nblk, hist, counts,
+                                             rows_cap, group_offsets, group_counts, row, k, token_of_row));
+  return moe::launch_status(what);
+}
+
+// The row copy into the groups and the zeroed padding rows, one launch.
+int launch_gather(const uint16_t *x, const int32_t *row, int T, int d, int E, int k, int64_t rows_cap,
+                  const int32_t *group_offsets, const int32_t *group_counts, uint16_t *x_perm,
+                  cudaStream_t s, const char *what) {
+  const int pad = E * kPadSplit;
+  MOE_LAUNCH("perm_gather", s, moe::launch_dep(perm_gather_kernel, pad + warp_grid(T), kThreads, 0, s, x, row, T, d, k,
+                                               rows_cap, pad, group_offsets, group_counts, x_perm));
+  return moe::launch_status(what);
+}
+
 }  // namespace
 
 namespace moe {
@@ -395,23 +466,12 @@ int moe_permute(const uint16_t *x, const int32_t *topk_idx, const int32_t *count
     return moe::set_error(MOE_ERR_ARG, "moe_permute: x/x_perm not 16-byte aligned");
   const moe::WsLayout L = moe::ws_layout(T, d, E, k, 0);
   if (ws_bytes < L.total) return moe::set_error(MOE_ERR_WORKSPACE, "moe_permute: workspace");
-  const int64_t A = int64_t(T) * k;
-  const int nblk = int(std::max<int64_t>(1, (A + kChunk - 1) / kChunk));
   int32_t *hist = reinterpret_cast<int32_t *>(static_cast<char *>(ws) + L.perm_hist);
-  MOE_LAUNCH("perm_hist", s, perm_hist_kernel<<<nblk, kThreads, 0, s>>>(topk_idx, A, E, nblk, hist));
-  if (int st = moe::launch_status("moe_permute: hist")) return st;
-  MOE_LAUNCH("perm_scan", s, perm_scan_kernel<<<1, 1024, 0, s>>>(hist, E, nblk, counts, rows_cap, group_offsets, group_counts));
-  if (int st = moe::launch_status("moe_permute: scan")) return st;
-  if (A > 0) {
-    MOE_LAUNCH("perm_rank", s, perm_rank_kernel<<<nblk, kThreads, 0, s>>>(topk_idx, A, E, nblk, hist, group_offsets, rows_cap,
-                                               row_of_assignment, k, nullptr));
-    if (int st = moe::launch_status("moe_permute: rank")) return st;
-    MOE_LAUNCH("perm_gather", s, perm_gather_kernel<<<warp_grid(T), kThreads, 0, s>>>(x, row_of_assignment, T, d, k, rows_cap,
-                                                         x_perm));
-    if (int st = moe::launch_status("moe_permute: gather")) return st;
-  }
-  MOE_LAUNCH("pad_zero", s, pad_zero_kernel<<<dim3(E, kPadSplit), kThreads, 0, s>>>(group_offsets, group_counts, E, d, rows_cap, x_perm));
-  return moe::launch_status("moe_permute: pad");
+  if (int st = launch_layout(topk_idx, int64_t(T) * k, E, hist, counts, rows_cap, group_offsets, group_counts,
+                             row_of_assignment, k, nullptr, s, "moe_permute: layout"))
+    return st;
+  return launch_gather(x, row_of_assignment, T, d, E, k, rows_cap, group_offsets, group_counts, x_perm,
+                       s, "moe_permute: gather");
 }
 
 int moe_permute_map(const int32_t *topk_idx, const int32_t *counts, int T, int E, int k,
@@ -432,19 +492,11 @@ int moe_permute_map(const int32_t *topk_idx, const int32_t *counts, int T, int E
   const moe::WsLayout L = moe::ws_layout(T, 8, E, k, 0);
   if (ws_bytes < L.perm_hist + size_t(E) * std::max<int64_t>(1, (int64_t(T) * k + kChunk - 1) / kChunk) * 4)
     return moe::set_error(MOE_ERR_WORKSPACE, "moe_permute_map: workspace");
-  const int64_t A = int64_t(T) * k;
-  const int nblk = int(std::max<int64_t>(1, (A + kChunk - 1) / kChunk));
   int32_t *hist = reinterpret_cast<int32_t *>(static_cast<char *>(ws) + L.perm_hist);
-  MOE_LAUNCH("perm_hist", s, perm_hist_kernel<<<nblk, kThreads, 0, s>>>(topk_idx, A, E, nblk, hist));
-  if (int st = moe::launch_status("moe_permute_map: hist")) return st;
-  MOE_LAUNCH("perm_scan", s, perm_scan_kernel<<<1, 1024, 0, s>>>(hist, E, nblk, counts, rows_cap, group_offsets, group_counts));
-  if (int st = moe::launch_status("moe_permute_map: scan")) return st;
-  if (A > 0) {
-    MOE_LAUNCH("perm_rank", s, perm_rank_kernel<<<nblk, kThreads, 0, s>>>(topk_idx, A, E, nblk, hist, group_offsets, rows_cap,
-                                               row_of_assignment, k, token_of_row));
-    if (int st = moe::launch_status("moe_permute_map: rank")) return st;
-  }
-  MOE_LAUNCH("pad_token", s, pad_token_kernel<<<E, kThreads, 0, s>>>(group_offsets, group_counts, E, rows_cap, token_of_row));
+  if (int st = launch_layout(topk_idx, int64_t(T) * k, E, hist, counts, rows_cap, group_offsets, group_counts,
+                             row_of_assignment, k, token_of_row, s, "moe_permute_map: layout"))
+    return st;
+  MOE_LAUNCH("pad_token", s, moe::launch_dep(pad_token_kernel, E, kThreads, 0, s, group_offsets, group_counts, E, rows_cap, token_of_row));
   return moe::launch_status("moe_permute_map: pad");
 }
 
@@ -458,7 +510,7 @@ int moe_unpermute_combine(const uint16_t *out_perm, const int32_t *row_of_assign
     return moe::set_error(MOE_ERR_ARG, "moe_unpermute_combine: null pointer");
   if (!moe::aligned16(out_perm) || !moe::aligned16(y))
     return moe::set_error(MOE_ERR_ARG, "moe_unpermute_combine: alignment");
-  MOE_LAUNCH("combine", s, combine_kernel<<<warp_grid(T), kThreads, 0, s>>>(out_perm, row_of_assignment, topk_gate, T, d, k, y));
+  MOE_LAUNCH("combine", s, moe::launch_dep(combine_kernel, warp_grid(T), kThreads, 0, s, out_perm, row_of_assignment, topk_gate, T, d, k, y));
   return moe::launch_status("moe_unpermute_combine: launch");
 }
 
@@ -479,26 +531,22 @@ int moe_unpermute_combine_bwd(const uint16_t *dy, const uint16_t *out_perm,
       (out_perm && !moe::aligned16(out_perm)))
     return moe::set_error(MOE_ERR_ARG, "moe_unpermute_combine_bwd: alignment");
   const int64_t rows_cap = moe_perm_rows_max(T, k, E);
-  if (T > 0) {
-    const int grid = warp_grid(T);
-    if (d_out_perm && d_gate) {
-      MOE_LAUNCH("combine_bwd", s, (combine_bwd_kernel<true, true><<<grid, kThreads, 0, s>>>(
-                                       dy, out_perm, row_of_assignment, topk_gate, T, d, k,
-                                       rows_cap, d_out_perm, d_gate)));
-    } else if (d_out_perm) {
-      MOE_LAUNCH("combine_bwd_dout", s, (combine_bwd_kernel<true, false><<<grid, kThreads, 0, s>>>(
-                                            dy, out_perm, row_of_assignment, topk_gate, T, d, k,
-                                            rows_cap, d_out_perm, d_gate)));
-    } else {
-      MOE_LAUNCH("combine_bwd_dgate", s, (combine_bwd_kernel<false, true><<<grid, kThreads, 0, s>>>(
-                                             dy, out_perm, row_of_assignment, topk_gate, T, d, k,
-                                             rows_cap, d_out_perm, d_gate)));
-    }
-    if (int st = moe::launch_status("moe_unpermute_combine_bwd: launch")) return st;
+  if (T == 0 && !d_out_perm) return MOE_OK;
+  const int pad = d_out_perm ? E * kPadSplit : 0, grid = pad + warp_grid(T);
+  if (d_out_perm && d_gate) {
+    MOE_LAUNCH("combine_bwd", s, moe::launch_dep(combine_bwd_kernel<true, true>, grid, kThreads, 0, s, dy, out_perm,
+                                                 row_of_assignment, topk_gate, T, d, k, rows_cap, pad,
+                                                 group_offsets, group_counts, d_out_perm, d_gate));
+  } else if (d_out_perm) {
+    MOE_LAUNCH("combine_bwd_dout", s, moe::launch_dep(combine_bwd_kernel<true, false>, grid, kThreads, 0, s, dy,
+                                                      out_perm, row_of_assignment, topk_gate, T, d, k, rows_cap,
+                                                      pad, group_offsets, group_counts, d_out_perm, d_gate));
+  } else {
+    MOE_LAUNCH("combine_bwd_dgate", s, moe::launch_dep(combine_bwd_kernel<false, true>, grid, kThreads, 0, s, dy,
+                                                       out_perm, row_of_assignment, topk_gate, T, d, k, rows_cap,
+                                                       pad, group_offsets, group_counts, d_out_perm, d_gate));
   }
-  if (!d_out_perm) return MOE_OK;
-  MOE_LAUNCH("pad_zero", s, pad_zero_kernel<<<dim3(E, kPadSplit), kThreads, 0, s>>>(group_offsets, group_counts, E, d, rows_cap, d_out_perm));
-  return moe::launch_status("moe_unpermute_combine_bwd: pad");
+  return moe::launch_status("moe_unpermute_combine_bwd: launch");
 }
 
 int moe_permute_bwd(const uint16_t *dx_perm, const int32_t *row_of_assignment,
@@ -521,11 +569,11 @@ int moe_permute_bwd(const uint16_t *dx_perm, const int32_t *row_of_assignment,
     if (!moe::aligned16(ws)) return moe::set_error(MOE_ERR_ARG, "moe_permute_bwd: ws alignment");
     w_t = reinterpret_cast<float *>(static_cast<char *>(ws) + L.w_router_t);
     dim3 grid((d + 31) / 32, (E + 31) / 32), block(32, 8);
-    MOE_LAUNCH("transpose_router", s, transpose_router_kernel<<<grid, block, 0, s>>>(w_router, d, E, w_t));
+    MOE_LAUNCH("transpose_router", s, moe::launch_dep(transpose_router_kernel, grid, block, 0, s, w_router, d, E, w_t));
     if (int st = moe::launch_status("moe_permute_bwd: transpose")) return st;
   }
-  MOE_LAUNCH("permute_bwd", s, permute_bwd_kernel<<<warp_grid(T), kThreads, 0, s>>>(dx_perm, row_of_assignment, topk_idx,
-                                                       d_logits, w_t, T, d, E, k, dx));
+  MOE_LAUNCH("permute_bwd", s, moe::launch_dep(permute_bwd_kernel, warp_grid(T), kThreads, 0, s, dx_perm,
+                                               row_of_assignment, topk_idx, d_logits, w_t, T, d, E, k, dx));
   return moe::launch_status("moe_permute_bwd: launch");
 }
 
@@ -641,22 +689,9 @@ extern "C" int moe_permute_noalloc(const uint16_t *x, const int32_t *topk_idx,
     return moe::set_error(MOE_ERR_ARG, "moe_permute_noalloc: x/x_perm not 16-byte aligned");
   int32_t *hist = nullptr;
   if (int st = noalloc_scratch(&hist)) return st;
-  const int nblk = int(nblk64);
-  MOE_LAUNCH("perm_hist", s, perm_hist_kernel<<<nblk, kThreads, 0, s>>>(topk_idx, A, E, nblk, hist));
-  if (int st = moe::launch_status("moe_permute_noalloc: hist")) return st;
-  MOE_LAUNCH("perm_scan", s, perm_scan_kernel<<<1, 1024, 0, s>>>(hist, E, nblk, counts, rows_cap,
-                                                                  group_offsets, group_counts));
-  if (int st = moe::launch_status("moe_permute_noalloc: scan")) return st;
-  if (A > 0) {
-    MOE_LAUNCH("perm_rank", s, perm_rank_kernel<<<nblk, kThreads, 0, s>>>(
-                                   topk_idx, A, E, nblk, hist, group_offsets, rows_cap,
-                                   row_of_assignment, k, nullptr));
-    if (int st = moe::launch_status("moe_permute_noalloc: rank")) return st;
-    MOE_LAUNCH("perm_gather", s, perm_gather_kernel<<<warp_grid(T), kThreads, 0, s>>>(
-                                     x, row_of_assignment, T, d, k, rows_cap, x_perm));
-    if (int st = moe::launch_status("moe_permute_noalloc: gather")) return st;
-  }
-  MOE_LAUNCH("pad_zero", s, pad_zero_kernel<<<dim3(E, kPadSplit), kThreads, 0, s>>>(group_offsets, group_counts, E,
-                                                                    d, rows_cap, x_perm));
-  return moe::launch_status("moe_permute_noalloc: pad");
+  if (int st = launch_layout(topk_idx, A, E, hist, counts, rows_cap, group_offsets, group_counts,
+                             row_of_assignment, k, nullptr, s, "moe_permute_noalloc: layout"))
+    return st;
+  return launch_gather(x, row_of_assignment, T, d, E, k, rows_cap, group_offsets, group_counts, x_perm,
+                       s, "moe_permute_noalloc: gather");
 }

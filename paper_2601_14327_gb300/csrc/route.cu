@@ -18,6 +18,7 @@ constexpr int kRouteThreads = 256;
 int padded_experts(int E) { return E <= 64 ? 64 : (E <= 128 ? 128 : (E <= 192 ? 192 : 256)); }
 
 __global__ void zero_i32_kernel(int32_t *p, int n) {
+  pdl_start();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0;
 }
 
@@ -110,10 +111,14 @@ int route_tokens_padded(int T) { return (T + kRtBK - 1) / kRtBK * kRtBK; }
 int route_dw_stride(int E) { return (route_tc_np(E) + 31) / 32 * 32; }
 
 // W [d, E] fp32 -> W3 [3][NP][d] bf16 (hi, mid, lo; rows e >= E are zero), by
-// 32 x 32 tiles transposed through shared memory.
+// 32 x 32 tiles transposed through shared memory. The first blocks also zero the counts that
+// the top-k kernel adds to (nullptr: none).
 __global__ void route_split_w_kernel(const float *__restrict__ w, int d, int E, int NP,
-                                     uint16_t *__restrict__ w3) {
+                                     uint16_t *__restrict__ w3, int32_t *__restrict__ counts) {
   __shared__ float tile[32][33];
+  pdl_start();
+  if (counts != nullptr && blockIdx.x == 0 && threadIdx.y == 0 && blockIdx.y * 32 + threadIdx.x < E)
+    counts[blockIdx.y * 32 + threadIdx.x] = 0;
   const int k0 = blockIdx.x * 32, e0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
   for (int i = ty; i < 32; i += 8) {
@@ -192,6 +197,7 @@ __global__ void __launch_bounds__(kRtThreads, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem_base = static_cast<uint32_t>(misc[0]);
+  pdl_start();  // TMEM is allocated; set-up overlaps the end of the previous kernel
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer ----
@@ -318,6 +324,7 @@ __global__ void __launch_bounds__(kRouteThreads, 4) route_topk_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int e = tid; e < NE; e += kRouteThreads) hist[e] = 0;
   __syncthreads();
+  pdl_start();
   for (int t = blockIdx.x * (kRouteThreads / 32) + warp; t < T;
        t += gridDim.x * (kRouteThreads / 32)) {
     float v[TK];
@@ -401,6 +408,7 @@ __global__ void load_stats_kernel(const int32_t *__restrict__ topk_idx, int64_t 
   __shared__ int hist[256];
   for (int e = threadIdx.x; e < E; e += blockDim.x) hist[e] = 0;
   __syncthreads();
+  pdl_start();
   for (int64_t a = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; a < A;
        a += int64_t(gridDim.x) * blockDim.x) {
     const int e = topk_idx[a];
@@ -426,6 +434,7 @@ __global__ void route_bwd_dz_kernel(const int32_t *__restrict__ topk_idx,
                                     const float *__restrict__ gate, const float *__restrict__ dgate,
                                     int T, int Tp, int k, int NP, float *__restrict__ d_logits,
                                     uint16_t *__restrict__ dz3) {
+  pdl_start();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= Tp) return;
   float g[8], dg[8], s = 0.f;
@@ -469,6 +478,7 @@ __global__ void route_bwd_dz_kernel(const int32_t *__restrict__ topk_idx,
 // dw_router[i, e] = sum over the splits, in order, of partial[split][i][e].
 __global__ void route_dw_reduce_kernel(const float *__restrict__ partial, int splits, int d,
                                        int E, int NE, float *__restrict__ dw_router) {
+  pdl_start();
   const int n = d * E;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
     const int i = idx / E, e = idx - i * E;
@@ -479,13 +489,14 @@ __global__ void route_dw_reduce_kernel(const float *__restrict__ partial, int sp
 }
 
 __global__ void zero_f32_kernel(float *p, int n) {
+  pdl_start();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0.f;
 }
 
 // Tensor-core logits: splits W into its three bf16 terms (w3), then one CTA per
 // (token tile, split). Returns the number of partial planes written in *splits.
 int launch_route_tc(const uint16_t *x, const float *w, int T, int d, int E, int NE, uint16_t *w3,
-                    float *partial, int *splits_out, cudaStream_t s) {
+                    float *partial, int32_t *counts, int *splits_out, cudaStream_t s) {
   const int NP = route_tc_np(E), MT = route_tc_mt(NP);
   const int stages = route_tc_stages(NP);
   const size_t smem = route_tc_smem(NP, stages, MT);
@@ -497,7 +508,7 @@ int launch_route_tc(const uint16_t *x, const float *w, int T, int d, int E, int 
     attr_set = true;
   }
   dim3 sgrid((d + 31) / 32, (NP + 31) / 32);
-  MOE_LAUNCH("route_split_w", s, route_split_w_kernel<<<sgrid, dim3(32, 8), 0, s>>>(w, d, E, NP, w3));
+  MOE_LAUNCH("route_split_w", s, moe::launch_dep(route_split_w_kernel, sgrid, dim3(32, 8), 0, s, w, d, E, NP, w3, counts));
   if (int st = moe::launch_status("moe_route: split router weight")) return st;
   CUtensorMap mx, mw;
   int st;
@@ -517,7 +528,7 @@ int launch_route_tc(const uint16_t *x, const float *w, int T, int d, int E, int 
   p.tmem_cols = route_tc_tmem_cols(NP, MT);
   p.partial = partial;
   dim3 grid((T + kRtBM * MT - 1) / (kRtBM * MT), splits);
-  MOE_LAUNCH("route_logits", s, route_tc_kernel<false><<<grid, kRtThreads, smem, s>>>(mx, mw, p));
+  MOE_LAUNCH("route_logits", s, moe::launch_dep(route_tc_kernel<false>, grid, kRtThreads, smem, s, mx, mw, p));
   *splits_out = splits;
   return moe::launch_status("moe_route: logits");
 }
@@ -528,14 +539,14 @@ int launch_route(const uint16_t *x, const float *w, const float *b, const uint8_
                  int32_t *counts, float *partial, uint16_t *w3, cudaStream_t s) {
   int splits = 0;
   if (lin == nullptr)
-    if (int st = launch_route_tc(x, w, T, d, E, NE, w3, partial, &splits, s)) return st;
+    if (int st = launch_route_tc(x, w, T, d, E, NE, w3, partial, counts, &splits, s)) return st;
   // one warp per token, grid-stride over the tokens; four blocks per SM, so that each
   // block's shared histogram sums ~100 tokens' assignments before its global atomics (one
   // block per 8 tokens sent 512k atomics to the counters at T=65536, top-8; the heaviest
   // expert's counter took ~60k of them one after another)
   const int grid2 = int(std::min<int64_t>((int64_t(T) + kRouteThreads / 32 - 1) / (kRouteThreads / 32),
                                           int64_t(moe::num_sms()) * 4));
-  MOE_LAUNCH("route_topk", s, route_topk_kernel<NE><<<grid2, kRouteThreads, 0, s>>>(
+  MOE_LAUNCH("route_topk", s, moe::launch_dep(route_topk_kernel<NE>, grid2, kRouteThreads, 0, s,
                                   partial, splits, lin, b, mask, T, E, k, lout, idx, gate, counts));
   return moe::launch_status("moe_route: top-k");
 }
@@ -586,8 +597,8 @@ int moe_route(const uint16_t *x, const float *w_router, const float *bias,
     partial = reinterpret_cast<float *>(static_cast<char *>(ws) + L.route_partial);
     w3 = reinterpret_cast<uint16_t *>(static_cast<char *>(ws) + L.route_w3);
   }
-  if (counts) {
-    MOE_LAUNCH("zero_counts", s, zero_i32_kernel<<<1, 256, 0, s>>>(counts, E));
+  if (counts && (logits_in || T == 0)) {  // else zeroed by the kernel that splits w_router
+    MOE_LAUNCH("zero_counts", s, moe::launch_dep(zero_i32_kernel, 1, 256, 0, s, counts, E));
     if (int st = moe::launch_status("moe_route: zero counts")) return st;
   }
   if (T == 0) return MOE_OK;
@@ -605,13 +616,13 @@ int moe_load_stats(const int32_t *topk_idx, int T, int k, int E, int32_t *counts
   if (E < 1 || E > 256 || k < 1 || T < 0) return moe::set_error(MOE_ERR_ARG, "moe_load_stats: sizes");
   if (!counts || (T > 0 && !topk_idx)) return moe::set_error(MOE_ERR_ARG, "moe_load_stats: null");
   if (!accumulate) {
-    MOE_LAUNCH("zero_counts", s, zero_i32_kernel<<<1, 256, 0, s>>>(counts, E));
+    MOE_LAUNCH("zero_counts", s, moe::launch_dep(zero_i32_kernel, 1, 256, 0, s, counts, E));
     if (int st = moe::launch_status("moe_load_stats: zero")) return st;
   }
   const int64_t A = int64_t(T) * k;
   if (A == 0) return MOE_OK;
   const int grid = int(std::min<int64_t>((A + 255) / 256, int64_t(moe::num_sms()) * 4));
-  MOE_LAUNCH("load_stats", s, load_stats_kernel<<<grid, 256, 0, s>>>(topk_idx, A, E, counts));
+  MOE_LAUNCH("load_stats", s, moe::launch_dep(load_stats_kernel, grid, 256, 0, s, topk_idx, A, E, counts));
   return moe::launch_status("moe_load_stats: launch");
 }
 
@@ -650,7 +661,7 @@ int launch_route_dw(const uint16_t *x, const uint16_t *dz3, int T, int d, int E,
   p.tmem_cols = route_tc_tmem_cols(NP, MT);
   p.partial = partial;
   dim3 grid((d + kRtBM * MT - 1) / (kRtBM * MT), splits);
-  MOE_LAUNCH("route_bwd_dw", s, route_tc_kernel<true><<<grid, kRtThreads, smem, s>>>(mx, mz, p));
+  MOE_LAUNCH("route_bwd_dw", s, moe::launch_dep(route_tc_kernel<true>, grid, kRtThreads, smem, s, mx, mz, p));
   *splits_out = splits;
   return moe::launch_status("moe_route_bwd: weight gradient");
 }
@@ -670,7 +681,7 @@ int moe_route_bwd(const uint16_t *x, const int32_t *topk_idx, const float *topk_
     return moe::set_error(MOE_ERR_ARG, "moe_route_bwd: alignment");
   if (T == 0) {
     const int n = d * E;
-    MOE_LAUNCH("zero_dw_router", s, zero_f32_kernel<<<std::min((n + 255) / 256, 1024), 256, 0, s>>>(dw_router, n));
+    MOE_LAUNCH("zero_dw_router", s, moe::launch_dep(zero_f32_kernel, std::min((n + 255) / 256, 1024), 256, 0, s, dw_router, n));
     return moe::launch_status("moe_route_bwd: zero");
   }
   const moe::WsLayout L = moe::ws_layout(T, d, E, k, 0);
@@ -679,13 +690,13 @@ int moe_route_bwd(const uint16_t *x, const int32_t *topk_idx, const float *topk_
   float *partial = reinterpret_cast<float *>(static_cast<char *>(ws) + L.route_dw_partial);
   const int NP = route_tc_np(E), Tp = route_tokens_padded(T);
   dim3 zgrid((Tp + 255) / 256, (NP + kDzExperts - 1) / kDzExperts);
-  MOE_LAUNCH("route_bwd_dz", s, route_bwd_dz_kernel<<<zgrid, 256, 0, s>>>(
+  MOE_LAUNCH("route_bwd_dz", s, moe::launch_dep(route_bwd_dz_kernel, zgrid, 256, 0, s,
                                     topk_idx, topk_gate, d_gate, T, Tp, k, NP, d_logits, dz3));
   if (int st = moe::launch_status("moe_route_bwd: dz")) return st;
   int splits = 0;
   if (int st = launch_route_dw(x, dz3, T, d, E, partial, &splits, s)) return st;
   const int n = d * E;
-  MOE_LAUNCH("route_bwd_reduce", s, route_dw_reduce_kernel<<<std::min((n + 255) / 256, 4 * moe::num_sms()), 256, 0, s>>>(
+  MOE_LAUNCH("route_bwd_reduce", s, moe::launch_dep(route_dw_reduce_kernel, std::min((n + 255) / 256, 4 * moe::num_sms()), 256, 0, s,
                                         partial, splits, d, E, route_dw_stride(E), dw_router));
   return moe::launch_status("moe_route_bwd: reduce");
 }

@@ -196,6 +196,24 @@ def test_permute_bit_exact(T, d, E, k, bias):
         assert (pad.float() == 0).all()
 
 
+@pytest.mark.parametrize("T,d,E,k", [(512, 64, 256, 8), (4096, 8, 1, 1),    # exactly one chunk of 4096
+                                     (4097, 72, 3, 1), (513, 264, 255, 8),  # one more
+                                     (1, 8, 8, 8), (3, 2048, 130, 5),
+                                     (12288, 16, 7, 1), (40000, 8, 33, 3)])
+def test_permute_chunk_edges(T, d, E, k):
+    """Layout and rows at the edges of the 4096-assignment chunks (one chunk takes a launch
+    less), of the expert table and of the 256-thread row loops; padding rows zero."""
+    rng = np.random.default_rng(T + E)
+    idx = np.argsort(rng.random((T, E)) ** 3, axis=1)[:, :k].astype(np.int32)
+    inp = {"x": torch.from_numpy(rng.standard_normal((T, d)).astype(np.float32)).to(torch.bfloat16)}
+    goff, gcnt, row, xp = _permute(inp, idx, E, k, counts=np.bincount(idx.reshape(-1), minlength=E))
+    ooff, ocnt, orow = O.permutation(idx, E, 128)
+    assert (goff == ooff).all() and (gcnt == ocnt).all() and (row == orow).all()
+    want = torch.zeros(int(ooff[-1]), d, dtype=torch.bfloat16)
+    want[torch.from_numpy(orow.reshape(-1)).long()] = inp["x"].repeat_interleave(k, dim=0)
+    assert torch.equal(xp[:int(ooff[-1])], want)
+
+
 def test_permute_all_tokens_one_expert_and_empty():
     T, d, E, k = 700, 128, 8, 1
     inp = case_inputs(T, d, E, k, 128, seed=2)
@@ -733,6 +751,39 @@ def test_fused_combine_without_tokens():
     torch.cuda.synchronize()
     assert b.y.shape == (0, 256) and (b.counts == 0).all()
 
+
+
+def test_back_to_back_steps_equal_synchronised_ones():
+    """Kernels start while their predecessors end (programmatic dependent launches): layer
+    steps of two shapes issued in turn with nothing waiting between, on one workspace each,
+    give the bits that each gives alone."""
+    names = ["y", "dx", "dw_gate_up", "dw_down", "dw_router", "topk_idx", "row_of_assignment",
+             "group_offsets", "d_logits", "counts"]
+
+    def state(T, d, E, k, F, seed):
+        inp = {n: v.cuda() for n, v in case_inputs(T, d, E, k, F, seed=seed).items()}
+        return layer.MoELayerBuffers(layer.LayerShape(T, d, E, k, F), "cuda"), inp
+
+    def step(s):
+        b, g = s
+        layer.forward(b, g["x"], g["w_router"], g["bias"], g["w_gate_up"], g["w_down"])
+        layer.backward(b, g["dy"], g["w_router"], g["w_gate_up"], g["w_down"])
+
+    states = [state(777, 256, 16, 4, 384, 1), state(5000, 384, 40, 3, 256, 2)]
+    want = []
+    for s in states:
+        step(s)
+        torch.cuda.synchronize()
+        want.append({n: getattr(s[0], n).clone() for n in names})
+    for s in states:
+        for n in names:
+            getattr(s[0], n).fill_(7)
+    for i in range(20):
+        step(states[i % 2])
+    torch.cuda.synchronize()
+    for s, w in zip(states, want):
+        for n in names:
+            assert torch.equal(getattr(s[0], n), w[n]), n
 
 
 def test_graph_replay_of_the_step_equals_eager():
