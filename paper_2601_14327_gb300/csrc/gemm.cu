@@ -624,6 +624,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 
 // ============================================================================
+// One-SM kernel above: activation GEMMs with few rows per expert (see act_plan) and the odd
+// last row blocks of large ones.
 // CTA-pair variant (cta_group::2): a cluster of two CTAs on two SMs computes a
 // 256 x BN tile. Each CTA stages its own 128 rows of A and half of B (BN/2 rows)
 // per k-block; one thread of the even CTA issues M=256 MMAs that read both CTAs'
@@ -1240,15 +1242,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 using moe::make_map;
 
-// The CTA-pair kernel runs every shape; MOE_GEMM_1SM=1 selects the one-SM kernel
-// instead (kept for A/B measurements of the two forms).
-template <int MODE> bool use_pair() {
-  static int v = -1;
-  if (v < 0) {
+// MOE_GEMM_1SM=1 selects the one-SM kernel and =0 the CTA-pair kernel for every GEMM, whatever
+// the shape (tests and A/B measurements of the two forms); -1: gemm_plan decides.
+int forced_one_sm() {
+  static int v = -2;
+  if (v == -2) {
     const char *e = getenv("MOE_GEMM_1SM");
-    v = (e && e[0] == '1') ? 0 : 1;
+    v = (e && (e[0] == '0' || e[0] == '1') && e[1] == 0) ? e[0] - '0' : -1;
   }
-  return v == 1;
+  return v;
 }
 
 // The CTA pairs claim tiles from a shared counter (Algorithm 2's greedy, online);
@@ -1385,6 +1387,36 @@ int64_t act_row_pairs(int64_t rows_cap, int E) {
   return std::max<int64_t>(0, rows_cap - int64_t(128) * E) / 256 + (E + 1) / 2;
 }
 
+// Kernel and column tile of an activation GEMM with N output columns and a reduction over K.
+// The CTA-pair kernel moves the least bytes per FLOP, but its tiles are 256 rows of one expert:
+// an expert with up to 128 rows leaves half of each tile unused, and a short list fills its
+// waves badly. The one-SM kernel has twice as many tiles of 128 rows to spread, at ~1.2 times
+// the time per k-block (96 KB of loads per CTA against 64 KB). With R = rows per expert on
+// average, one-SM up to R = 640 and R * K = 3 * 2^18 (a long reduction makes the loads weigh
+// more than the tile counts). Measured over 134 GEMMs of 34 random layers (R 0.2-1,500, K
+// 256-7168, N 256-7168), against the pair kernel: 0.87 of its time on average, 0.53 at best
+// (10 us class), 1.08 at worst (12.4 -> 13.4 us). On both sides of the line: pair 121 us / one-SM
+// 134 us at R = 304, K = 6528; 187 / 205 us at R = 1492, K = 6912; 91 / 92 us at R = 580,
+// K = 1536; 155 / 143 us at R = 40, K = 2304.
+// Its column tile is 128 wide where that takes less in waves of one tile per SM, a 128-wide tile
+// counted as 0.65 of a 256-wide one (at R = 25: 146 us in 256-wide and 121 us in 128-wide tiles
+// for N = 384, K = 7168; at R = 549: 9.6 and 12.0 us for N = 384, K = 768).
+struct GemmPlan {
+  bool pair;
+  int bn;
+};
+GemmPlan act_plan(bool gate_up, int N, int K, int64_t rows_cap, int E) {
+  const int64_t A = std::max<int64_t>(0, rows_cap - int64_t(128) * E);  // T * k
+  const int forced = forced_one_sm();
+  if (forced >= 0 || A > int64_t(640) * E || A * K > (int64_t(3) << 18) * E)
+    return {forced != 1, gate_up ? 256 : tile_cols(N, act_row_pairs(rows_cap, E))};
+  if (gate_up || N < 256) return {false, gate_up ? 256 : 128};
+  // row blocks: full ones and three quarters of one more per expert that can have rows
+  const int64_t blocks = A / 128 + (3 * std::min<int64_t>(E, A) + 3) / 4, sms = moe::num_sms();
+  auto waves = [&](int bn) { return (blocks * ((N + bn - 1) / bn) + sms - 1) / sms; };
+  return {false, 13 * waves(128) < 20 * waves(256) ? 128 : 256};
+}
+
 // Builds the tensor maps for one GEMM and launches it. A: [a_rows, a_cols] row-major
 // bf16; B likewise. N = output columns (for kGateUp: 2F, in tiles of 128 gate + 128 up).
 // The output p.out is [o_rows, o_cols] row-major bf16.
@@ -1408,14 +1440,15 @@ int run_gemm_out(int N, const void *a_base, uint64_t a_rows, uint64_t a_cols, co
                  uint64_t b_rows, uint64_t b_cols, const void *o_base, uint64_t o_rows,
                  uint64_t o_cols, GemmParams p, cudaStream_t s, const char *what) {
   using Tr = Traits<MODE>;
-  const bool pair = use_pair<MODE>();
   if (!Tr::WGRAD) p.dynamic = 0;  // equal-cost tiles: fixed stride, no counter to reset
-  const int BN = MODE == kGateUp ? 256
-                                 : tile_cols(N, Tr::WGRAD ? int64_t(p.E) * ((p.m_tiles_w + 1) / 2)
-                                                          : act_row_pairs(int64_t(a_rows), p.E));
+  const bool gather = p.token_of_row != nullptr;
+  const GemmPlan plan = Tr::WGRAD || gather
+                            ? GemmPlan{forced_one_sm() != 1, MODE == kGateUp ? 256 : tile_cols(N, int64_t(p.E) * ((p.m_tiles_w + 1) / 2))}
+                            : act_plan(MODE == kGateUp, N, p.nkb * BK, int64_t(a_rows), p.E);
+  const bool pair = plan.pair;
+  const int BN = plan.bn;
   p.n_tiles = (N + BN - 1) / BN;
   p.n_cols = N;
-  const bool gather = p.token_of_row != nullptr;
   if (gather && MODE != kGateUp && MODE != kWgradGateUp)
     return moe::set_error(MOE_ERR_UNSUPPORTED, "%s: no gathered operand in this GEMM", what);
   if (gather && !pair)
@@ -1799,7 +1832,7 @@ int moe_grouped_ffn_bwd_dgrad(const uint16_t *d_out_perm, const uint16_t *ab_sav
   p.out = d_ab;
   p.aux = ab_saved;
   if (gate) {
-    const int cols = tile_cols(F, act_row_pairs(rows_cap, E));
+    const int cols = act_plan(false, F, d, rows_cap, E).bn;  // the dH GEMM's column tile
     gate_stride = 2 * ((F + cols - 1) / cols);  // column halves of the N tiles
     p.gate_partial = reinterpret_cast<float *>(static_cast<char *>(ws) + L.gate_partial);
     p.gate_stride = gate_stride;

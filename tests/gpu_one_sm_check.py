@@ -1,6 +1,7 @@
 """Child-process check of the one-SM GEMM kernel (selected by MOE_GEMM_1SM=1, which
-the library reads once per process): layer cases through the C ABI against the
-oracle. Run by test_gpu_parity.py::test_one_sm_gemm_kernel_against_oracle."""
+the library reads once per process) or of the CTA-pair kernel (=0): layer cases through
+the C ABI against the oracle. Run by
+test_gpu_parity.py::test_one_sm_gemm_kernel_against_oracle."""
 import os
 import sys
 
@@ -44,7 +45,8 @@ def check(T, d, E, k, F, n_masked):
 
 
 if __name__ == "__main__":
-    assert os.environ.get("MOE_GEMM_1SM") == "1"
-    check(1500, 384, 12, 4, 640, 3)  # ragged groups, N tiles of 128, empty experts
+    assert os.environ.get("MOE_GEMM_1SM") in ("0", "1")
+    check(1500, 384, 12, 4, 640, 3)  # ragged groups, N not a multiple of 256, empty experts
     check(700, 512, 8, 8, 256, 0)    # k = number of experts
-    print("one-SM GEMM kernel: ok")
+    check(3000, 256, 256, 8, 256, 40)  # the maximum expert count
+    print("GEMM kernel: ok")

@@ -299,12 +299,16 @@ def test_layer_fwd_bwd_against_oracle(T, d, E, k, F, bias, n_masked):
 
 
 @pytest.mark.parametrize("T,d,E,k,F,bias,n_masked", [
-    # >= 3 waves of 256-wide tiles with a cut last one: in every GEMM whose N is 384 or 640
-    (6000, 384, 64, 4, 640, "zipf", 5),
-    # the same with 1 of 2 column tiles cut, one-block groups and empty experts
+    # CTA pairs (900 rows per expert), >= 3 waves of 256-wide tiles with a cut last one in
+    # every GEMM whose N is 384 or 640
+    (9000, 384, 40, 4, 640, "zipf", 5),
+    # one-SM activation GEMMs, cut 256-wide tiles, one-block groups and empty experts; CTA-pair
+    # weight gradients with cut tiles
     (5000, 640, 128, 3, 384, "loguniform", 0),
-    # 256-wide tiles would not fill half the CTA pairs: 128-wide ones, N a multiple of 256
+    # one wave either way: 128-wide tiles, N a multiple of 256
     (200, 256, 3, 2, 512, "none", 0),
+    # CTA pairs (667 rows per expert), lists too short for 256-wide tiles
+    (1000, 256, 3, 2, 512, "none", 0),
 ])
 def test_column_tile_widths_against_oracle(T, d, E, k, F, bias, n_masked):
     test_layer_fwd_bwd_against_oracle(T, d, E, k, F, bias, n_masked)
@@ -468,11 +472,13 @@ def test_gathered_layer_equals_materialized(T, d, E, k, F, n_masked):
     assert (ua[rr] == ub[rr]).all()
 
 
-def test_one_sm_gemm_kernel_against_oracle():
-    """The one-SM GEMM kernel (MOE_GEMM_1SM=1, kept for A/B measurements against the
-    CTA-pair kernel) on layer cases; the variable is read once per process, so the
+@pytest.mark.parametrize("one_sm", ["1", "0"])
+def test_one_sm_gemm_kernel_against_oracle(one_sm):
+    """The one-SM GEMM kernel in every GEMM (MOE_GEMM_1SM=1), and the CTA-pair kernel in
+    every GEMM (=0; by default these few rows per expert take the one-SM kernel in the
+    activation GEMMs), on layer cases; the variable is read once per process, so the
     cases run in a child process."""
-    env = dict(os.environ, MOE_GEMM_1SM="1")
+    env = dict(os.environ, MOE_GEMM_1SM=one_sm)
     script = os.path.join(os.path.dirname(os.path.abspath(__file__)), "gpu_one_sm_check.py")
     r = subprocess.run([sys.executable, script], env=env, capture_output=True, text=True,
                        timeout=900)
