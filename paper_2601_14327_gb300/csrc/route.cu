@@ -14,7 +14,7 @@ MOE_DEV_ERR_DECL
 
 namespace {
 
-constexpr int kRouteThreads = 256;
+constexpr int kTopkThreads = 128;
 int padded_experts(int E) { return E <= 64 ? 64 : (E <= 128 ? 128 : (E <= 192 ? 192 : 256)); }
 
 __global__ void zero_i32_kernel(int32_t *p, int n) {
@@ -28,10 +28,10 @@ __global__ void zero_i32_kernel(int32_t *p, int n) {
 // Henry, Tang and Heinecke, "Leveraging the bfloat16 artificial intelligence
 // datatype for higher-precision computations", 2019). Three 8-bit significands
 // cover the 24 of a normal fp32 weight, every bf16 x bf16 product is exact in
-// fp32, and the three MMAs of each k-step accumulate into one fp32 accumulator
-// in tensor memory, so the logits carry fp32 accumulation error only.
+// fp32 and accumulates in fp32 in tensor memory, so the logits carry fp32
+// accumulation error only.
 //
-// One CTA = one 128-token tile x one range of k-blocks (a split of the
+// One CTA = one or two 128-token tiles x one range of k-blocks (a split of the
 // reduction over d when there are fewer tiles than CTA slots). Warp 0 issues the
 // TMA loads (x tile + the three weight terms per k-block), warp 1 owns TMEM and
 // issues the MMAs, then all four warps read the accumulator (one TMEM lane
@@ -43,7 +43,8 @@ constexpr int kRtBK = 64;        // k-block: 64 bf16 = one 128-byte swizzle row
 constexpr int kRtThreads = 128;
 constexpr int kRtSms = 152;           // SMs of a GB300: the splits aim to fill them
 constexpr int kRtSmemPerSm = 233472;  // shared memory per SM (228 KB)
-constexpr int kRtMaxSplits = 8;
+constexpr int kRtLogitsSplits = 8;
+constexpr int kRtDwSplits = 64;
 constexpr uint32_t kRtABytes = kRtBM * kRtBK * 2;
 constexpr int kRtMaxSmem = 232448;  // opt-in dynamic shared memory per CTA
 constexpr uint64_t kRtWaitNs = 2000000000ull;
@@ -53,7 +54,7 @@ struct RouteTcParams {
   int MT;            // 128-row tiles per CTA (1 or 2); tile m's accumulator at TMEM column 256*m
   int kb_per_split;  // k-blocks of one split
   int nkb;           // k-blocks of the reduction (over d, or over the padded tokens)
-  int NP;            // MMA N: experts rounded up to 16
+  int NP;            // experts rounded up to 16
   int NE;            // row stride of the partial logits
   int stages;        // shared-memory ring depth
   uint32_t tmem_cols;
@@ -62,47 +63,90 @@ struct RouteTcParams {
 
 // Experts rounded up to the MMA's N granularity, and the matching TMEM allocation.
 int route_tc_np(int E) { return (E + 15) / 16 * 16; }
-// 128-row tiles per CTA: two above 96 experts (up to 192), where the three weight terms of a
-// k-block (3 x NP x 128 bytes) outweigh the 16 KB x tile: two x tiles share each weight stage,
-// halving the L2 reads of the weight terms per FLOP; one CTA per SM either way.
-int route_tc_mt(int NP) { return (NP > 96 && NP <= 192) ? 2 : 1; }
-uint32_t route_tc_tmem_cols(int NP, int MT) {
+// Terms of the second operand (the weight, or dZ) per MMA. Logits: 1, each k-step adds the hi, mid
+// and lo products to one accumulator. x^T dZ: as many as fit along N (256), each with an accumulator of
+// its own, added at the end; the x tile is then read from shared memory once (up to 80 experts)
+// or twice (up to 128) per k-step instead of three times, and shared memory sets the pace of
+// these short-N MMAs: 43 / 31 us at T=16384, d=4096, 64 experts, 47 / 40 us at T=35700, d=2856, 57.
+int route_dw_group(int NP) { return std::min(3, 256 / NP); }
+uint32_t route_tc_tmem_cols(int c, int MT) {  // c: accumulator columns of one tile
   if (MT == 2) return 512u;
-  return NP <= 32 ? 32u : (NP <= 64 ? 64u : (NP <= 128 ? 128u : 256u));
+  return c <= 32 ? 32u : (c <= 64 ? 64u : (c <= 128 ? 128u : 256u));
 }
-uint32_t route_tc_stage_bytes(int NP, int MT = 1) {
-  return uint32_t(MT) * kRtABytes + 3u * uint32_t(NP) * 128u;
-}
-size_t route_tc_smem(int NP, int stages, int MT = 1) {
+uint32_t route_tc_stage_bytes(int NP, int MT) { return uint32_t(MT) * kRtABytes + 3u * uint32_t(NP) * 128u; }
+size_t route_tc_smem(int NP, int stages, int MT) {
   return 1024 + size_t(stages) * route_tc_stage_bytes(NP, MT) + size_t(2 * stages + 1) * 8 + 16;
 }
-// Two CTAs per SM with a ring of at least two stages each where that fits (more
-// independent x streams per SM: measured faster than one CTA with a deeper ring), else
-// one CTA per SM with the deepest ring that fits.
-bool route_tc_two_per_sm(int NP) {
-  return 2 * (route_tc_smem(NP, 2) + 1024) <= size_t(kRtSmemPerSm);
+// CTAs per SM and ring depth: with one 128-row tile per CTA, two CTAs per SM if a ring of at
+// least two stages each fits (more independent x streams per SM: measured faster than one
+// CTA with a deeper ring); else one with the deepest ring that fits (0 stages: none of two).
+void route_tc_ring(int NP, int MT, int *per_sm, int *stages) {
+  *per_sm = MT == 1 && 2 * (route_tc_smem(NP, 2, 1) + 1024) <= size_t(kRtSmemPerSm) ? 2 : 1;
+  int st = 0;
+  while (st < 8 && (*per_sm == 2 ? 2 * (route_tc_smem(NP, st + 1, 1) + 1024) <= size_t(kRtSmemPerSm)
+                                 : int64_t(st + 1) * route_tc_stage_bytes(NP, MT) <= kRtMaxSmem - 2048))
+    ++st;
+  *stages = st >= 2 ? st : 0;
 }
-int route_tc_stages(int NP) {
-  int st = 2;
-  if (route_tc_two_per_sm(NP)) {
-    while (st < 8 && 2 * (route_tc_smem(NP, st + 1) + 1024) <= size_t(kRtSmemPerSm)) ++st;
-  } else {
-    st = int((kRtMaxSmem - 2048) / route_tc_stage_bytes(NP, route_tc_mt(NP)));
-  }
-  return std::min(8, st);
-}
-// Splits of the reduction: enough CTAs to fill the SMs' CTA slots when the M rows (tokens
-// for the logits, d_model for the weight gradient) give few tiles. A function of
-// (M, K, NP) alone, so the workspace size is too. K > 0.
-void route_tc_split(int M, int K, int NP, int *splits, int *kb_per_split) {
-  const int rows = kRtBM * route_tc_mt(NP);
-  const int tiles = std::max(1, (M + rows - 1) / rows);
+
+struct RtPlan {
+  int MT;  // 128-row tiles per CTA
+  int stages, splits, kb_per_split;
+};
+// Logits, M tokens over K = d. Two tiles per CTA from 97 to 192 experts, where the three weight
+// terms of a k-block (3 x NP x 128 bytes) outweigh the 16 KB x tile: two x tiles share each
+// weight stage. Splits: enough CTAs to fill the SMs' CTA slots when the tokens give few tiles. The
+// plan fixes the order in which a logit's products are summed, and with it the last bits that
+// decide a near tie: it is a function of (M, K, NP) alone, and a change of it can route a token
+// differently.
+RtPlan route_logits_plan(int M, int K, int NP) {
+  RtPlan r;
+  int per_sm;
+  r.MT = NP > 96 && NP <= 192 ? 2 : 1;
+  route_tc_ring(NP, r.MT, &per_sm, &r.stages);
+  const int rows = kRtBM * r.MT, tiles = std::max(1, (M + rows - 1) / rows);
   const int nkb = (K + kRtBK - 1) / kRtBK;
-  const int target = kRtSms * (route_tc_two_per_sm(NP) ? 2 : 1);
-  int s = std::max(1, std::min({target / tiles, kRtMaxSplits, nkb}));
-  const int per = (nkb + s - 1) / s;
-  *kb_per_split = per;
-  *splits = (nkb + per - 1) / per;  // every split gets at least one k-block
+  const int s = std::max(1, std::min({kRtSms * per_sm / tiles, kRtLogitsSplits, nkb}));
+  r.kb_per_split = (nkb + s - 1) / s;
+  r.splits = (nkb + r.kb_per_split - 1) / r.kb_per_split;  // every split gets at least one k-block
+  return r;
+}
+// x^T dZ, M = d features over K tokens: the tiles per CTA and splits of the reduction with the
+// least estimated time (ns). An SM takes a k-block of a CTA in the longest of its share of the HBM
+// rate for the x tiles, its shared-memory traffic (TMA writes, MMA reads) at ~243 B/ns, and, with
+// few CTAs, a load's way through the ring (~2.3 us for load, wait and MMA over the stages); a
+// split adds its partial sums' write and read. A function of (M, K, NP) alone, so the workspace
+// size is too. K > 0. Measured, with the logits' plan (at most 8 splits) / with this one: 30 /
+// 12.6 us at T=22360, d=1128, 28 experts (9 tiles: 72 CTAs / 32 splits), 67 / 40 us at T=35700,
+// d=2856, 57 experts, 22.9 / 18.0 us at T=3516, d=3328, 167 experts; both 49 us at T=8191, d=7168, 171.
+RtPlan route_dw_plan(int M, int K, int NP) {
+  const int nkb = (K + kRtBK - 1) / kRtBK;
+  const int group = route_dw_group(NP), mmas = (3 + group - 1) / group;
+  const int64_t ne = (NP + 31) / 32 * 32;
+  RtPlan best{1, 2, 1, nkb};
+  int64_t best_ns = INT64_MAX;
+  for (int mt = 1; mt <= (M > kRtBM ? 2 : 1); ++mt) {
+    int per_sm, stages;
+    route_tc_ring(NP, mt, &per_sm, &stages);
+    if (stages == 0) continue;
+    const int64_t tiles = std::max(1, (M + kRtBM * mt - 1) / (kRtBM * mt));
+    const int64_t a = int64_t(mt) * kRtABytes, w = int64_t(3) * NP * 128;
+    const int64_t busy = std::max<int64_t>(a * 1000 / 44700, (a + w + mmas * a + mt * w) * 1000 / 243000);
+    const int64_t ring = 2300 / stages, slots = int64_t(kRtSms) * per_sm;
+    for (int s = 1; s <= std::min(nkb, kRtDwSplits); ++s) {
+      const int per = (nkb + s - 1) / s;
+      if ((nkb + per - 1) / per != s) continue;  // every split gets at least one k-block
+      const int64_t full = tiles * s / slots, rest = tiles * s % slots;
+      int64_t ns = full * (per * std::max(per_sm * busy, ring) + 1500);
+      if (rest > 0) ns += per * std::max(rest > kRtSms ? 2 * busy : busy, ring) + 1500;
+      if (s > 1) ns += s * int64_t(M) * ne * 8 / 4000;
+      if (ns < best_ns) {
+        best_ns = ns;
+        best = {mt, stages, s, per};
+      }
+    }
+  }
+  return best;
 }
 
 // Router weight gradient: tokens padded to one k-block, and the row stride of its
@@ -147,7 +191,9 @@ __global__ void route_split_w_kernel(const float *__restrict__ w, int d, int E, 
 // DW = true: the router weight gradient, partial[split][i][e] = sum over the split's
 // tokens t of x[t, i] * dZ[t, e] (A = x^T, read MN-major from x itself as two 64 x 64
 // boxes per k-block; B = dZ's three bf16 terms, K-major [3][NP][T padded to 64]).
-template <bool DW>
+// G = terms per MMA (see route_dw_group), at compile time: the issuing thread's loop sets the pace
+// otherwise (with a bound read from the parameters 110 instead of 79 us at T=32768, 128 experts).
+template <bool DW, int G>
 __global__ void __launch_bounds__(kRtThreads, 1)
     route_tc_kernel(const __grid_constant__ CUtensorMap tmX,
                     const __grid_constant__ CUtensorMap tmW, const RouteTcParams p) {
@@ -171,10 +217,13 @@ __global__ void __launch_bounds__(kRtThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mt = blockIdx.x, split = blockIdx.y;
   const int kb0 = split * p.kb_per_split, nk = min(p.nkb, kb0 + p.kb_per_split) - kb0;
-  // Each tile starts its k-loop at its own offset, so that the CTAs do not all read
-  // the same weight tile from L2 at the same time (the order is fixed per tile).
-  const int rot = nk > 0 ? int((mt * 7u) % uint32_t(nk)) : 0;
-  const uint32_t idesc = tc::idesc_bf16_f32(kRtBM, p.NP, DW, false);
+  // Each token tile starts its k-loop at its own offset, so that the CTAs do not all read
+  // the same weight tile from L2 at the same time (the order is fixed per tile; without it
+  // 88 instead of 71 us at T=26750, d=4296, 61 experts). x^T dZ's feature tiles read slices
+  // of the same token rows and stay in step (48 against 51 us at T=35700, d=2856).
+  const int rot = !DW && nk > 0 ? int((mt * 7u) % uint32_t(nk)) : 0;
+  const uint32_t idesc_g = tc::idesc_bf16_f32(kRtBM, G * p.NP, DW, false);
+  const uint32_t idesc_1 = tc::idesc_bf16_f32(kRtBM, p.NP, DW, false);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -250,18 +299,18 @@ __global__ void __launch_bounds__(kRtThreads, 1)
       }
       tc::fence_after_sync();
       const uint32_t a_s = s0 + s * stage_bytes, b_s = a_s + a_bytes;
+      // (a descriptor's address field counts 16 bytes: steps are plain additions)
+      const uint64_t b0 = tc::smem_desc_sw128(b_s, 16, 1024);
       for (int m = 0; m < p.MT; ++m) {
-        const uint32_t am = a_s + uint32_t(m) * kRtABytes;
+        const uint32_t am = a_s + uint32_t(m) * kRtABytes, d = tmem_base + uint32_t(m) * 256u;
+        const uint64_t a0 = DW ? tc::smem_desc_sw128(am, 8192, 1024) : tc::smem_desc_sw128(am, 16, 1024);
 #pragma unroll
         for (int kk = 0; kk < kRtBK / 16; ++kk) {
-          const uint64_t ad = DW ? tc::smem_desc_sw128(am + kk * 2048, 8192, 1024)
-                                 : tc::smem_desc_sw128(am + kk * 32, 16, 1024);
+          const uint64_t ad = a0 + uint64_t(DW ? kk * 128 : kk * 2);
+          tc::mma_bf16(d, ad, b0 + uint64_t(kk * 2), idesc_g, (it != 0 || kk != 0) ? 1u : 0u);
 #pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            const uint64_t bd = tc::smem_desc_sw128(b_s + j * b_bytes + kk * 32, 16, 1024);
-            tc::mma_bf16(tmem_base + uint32_t(m) * 256u, ad, bd, idesc,
-                         (it != 0 || kk != 0 || j != 0) ? 1u : 0u);
-          }
+          for (int j = G; j < 3; ++j)  // terms that did not fit: into the first accumulator
+            tc::mma_bf16(d, ad, b0 + uint64_t(kk * 2) + uint64_t(j) * (b_bytes >> 4), idesc_1, 1u);
         }
       }
       tc::mma_commit(empty_bar(s));
@@ -289,10 +338,17 @@ __global__ void __launch_bounds__(kRtThreads, 1)
       float *dst = p.partial + (size_t(split) * p.M + t) * p.NE;
       for (int c0 = 0; c0 < p.NP; c0 += 32) {
         uint32_t r[32];
-        tc::tmem_ld_32x32b_x32(tmem_base + (uint32_t(warp * 32) << 16) + uint32_t(m) * 256u +
-                                   uint32_t(c0),
-                               r);
+        const uint32_t tb = tmem_base + (uint32_t(warp * 32) << 16) + uint32_t(m) * 256u + uint32_t(c0);
+        tc::tmem_ld_32x32b_x32(tb, r);
         tc::tmem_ld_wait();
+#pragma unroll
+        for (int j = 1; j < G; ++j) {
+          uint32_t q[32];
+          tc::tmem_ld_32x32b_x32(tb + uint32_t(j * p.NP), q);
+          tc::tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(q[i]));
+        }
         if (t < p.M) {
 #pragma unroll
           for (int q = 0; q < 8; ++q)
@@ -309,97 +365,193 @@ __global__ void __launch_bounds__(kRtThreads, 1)
   }
 }
 
-// One warp per token: logits = sum of the split
-// partials (fixed order) + bias, pruned experts -inf, k rounds of a warp arg-max
-// (ties to the lower index), softmax over the selected logits, per-expert
-// histogram (shared per block, then one global add per expert and block).
-template <int NE>
-__global__ void __launch_bounds__(kRouteThreads, 4) route_topk_kernel(
-    const float *__restrict__ partial, int splits, const float *__restrict__ logits_in,
+// The K largest (key, expert) pairs so far, descending; equal keys by ascending expert.
+template <int K> struct TopList {
+  unsigned key[K];  // order-preserving key of a logit, 0: empty
+  int e[K];
+  __device__ __forceinline__ TopList() {
+#pragma unroll
+    for (int s = 0; s < K; ++s) {
+      key[s] = 0u;
+      e[s] = -1;
+    }
+  }
+  // Experts come in ascending order: a later one passes strictly smaller keys only (the
+  // entries from there on move down one slot).
+  __device__ __forceinline__ void add(unsigned x, int xe) {
+    bool up = false;
+#pragma unroll
+    for (int s = 0; s < K; ++s) {
+      up = up || x > key[s];
+      const unsigned lk = up ? key[s] : x;
+      const int le = up ? e[s] : xe;
+      key[s] = up ? x : key[s];
+      e[s] = up ? xe : e[s];
+      x = lk;
+      xe = le;
+    }
+  }
+  static __device__ __forceinline__ bool before(unsigned ka, int ea, unsigned kb, int eb) {
+    return ka > kb || (ka == kb && ea < eb);
+  }
+  // The K largest of this list and lane ^ `lane_xor`'s: the larger of entry s here and entry
+  // K-1-s there are those K, as a bitonic sequence, which log2(K) exchange stages sort.
+  __device__ __forceinline__ void merge(int lane_xor) {
+    unsigned ok[K];
+    int oe[K];
+#pragma unroll
+    for (int s = 0; s < K; ++s) {
+      ok[s] = __shfl_xor_sync(0xffffffffu, key[s], lane_xor);
+      oe[s] = __shfl_xor_sync(0xffffffffu, e[s], lane_xor);
+    }
+#pragma unroll
+    for (int s = 0; s < K; ++s) {
+      const bool other = before(ok[K - 1 - s], oe[K - 1 - s], key[s], e[s]);
+      key[s] = other ? ok[K - 1 - s] : key[s];
+      e[s] = other ? oe[K - 1 - s] : e[s];
+    }
+#pragma unroll
+    for (int h = K / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int s = 0; s < K; ++s)
+        if ((s & h) == 0) {
+          const bool sw = before(key[s + h], e[s + h], key[s], e[s]);
+          const unsigned ka = key[s], kb = key[s + h];
+          const int ea = e[s], eb = e[s + h];
+          key[s] = sw ? kb : ka;
+          e[s] = sw ? eb : ea;
+          key[s + h] = sw ? ka : kb;
+          e[s + h] = sw ? ea : eb;
+        }
+  }
+};
+
+// LPT (4 or 16) lanes per token: logits = sum of the split partials (fixed order) + bias, pruned
+// experts -inf; top-k (ties to the lower index), softmax over the selected logits,
+// per-expert histogram (shared per block, then one global add per expert and block).
+// Lane q keeps the K largest logits of experts 4 LPT i + 4 q .. + 3 in registers (~5 K
+// instructions per logit, 32 / LPT tokens per instruction), exchanges merge the lists.
+// Issue-bound with many tokens: 4 lanes, ~250 warp instructions per token at 128 experts, top-8,
+// against ~1,000 for a warp per token with two redux per selected expert: 21 us instead of 40
+// at T=32768 (the compares and selects, at half the issue rate, are its bound now). Latency-bound
+// with few: 16 lanes, a quarter of the chain per lane.
+template <int K, int LPT>
+__global__ void __launch_bounds__(kTopkThreads) route_topk_kernel(
+    const float *__restrict__ partial, int splits, int NE, const float *__restrict__ logits_in,
     const float *__restrict__ bias, const uint8_t *__restrict__ active_mask, int T, int E, int k,
     float *__restrict__ logits_out, int32_t *__restrict__ topk_idx, float *__restrict__ topk_gate,
     int32_t *__restrict__ counts) {
-  constexpr int TK = NE / 32;  // logits per lane
-  __shared__ int hist[NE];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int e = tid; e < NE; e += kRouteThreads) hist[e] = 0;
-  __syncthreads();
+  __shared__ int hist[256];
+  __shared__ __align__(16) float s_bias[256];
+  __shared__ uint8_t s_live[256];
+  const int tid = threadIdx.x, q = tid % LPT;
+  for (int e = tid; e < 256; e += kTopkThreads) hist[e] = 0;
   pdl_start();
-  for (int t = blockIdx.x * (kRouteThreads / 32) + warp; t < T;
-       t += gridDim.x * (kRouteThreads / 32)) {
-    float v[TK];
+  for (int e = tid; e < 256; e += kTopkThreads) {
+    s_bias[e] = (bias != nullptr && e < E) ? bias[e] : 0.f;
+    s_live[e] = e < E && (active_mask == nullptr || active_mask[e] != 0);
+  }
+  __syncthreads();
+  constexpr int per_block = kTopkThreads / LPT;
+  // (whole warps stay in the loop: the merges are warp-wide)
+  for (int t0 = blockIdx.x * per_block; t0 < T; t0 += gridDim.x * per_block) {
+    const int t = t0 + tid / LPT;
+    const bool mine = t < T;
+    TopList<K> top;
+    // four chunks of four experts at a time, so that their loads (of up to four partials each)
+    // are in flight together
+    for (int g0 = 0; g0 < E; g0 += 16 * LPT) {
+      float z[4][4] = {};
+      if (mine) {
+        if (logits_in != nullptr) {
 #pragma unroll
-    for (int j = 0; j < TK; ++j) {
-      const int e = lane + 32 * j;
-      float z = 0.f;
-      if (logits_in != nullptr) {
-        z = e < E ? logits_in[size_t(t) * E + e] : 0.f;
-      } else {
-        for (int y = 0; y < splits; ++y) z += partial[(size_t(y) * T + t) * NE + e];
-        if (bias != nullptr && e < E) z += bias[e];
-      }
-      if (e >= E || (active_mask != nullptr && active_mask[e] == 0)) z = -INFINITY;
-      v[j] = z;
-      if (logits_out != nullptr && e < E) logits_out[size_t(t) * E + e] = z;
-    }
-    // Order-preserving unsigned keys of the logits (a larger float gives a larger key,
-    // -0 is taken as +0 so that equal logits tie; 0 marks an expert that cannot be
-    // selected). Each round takes the warp maximum of the keys with one redux and the
-    // lowest expert holding it with a second: a lane offers expert 32 j + lane for its
-    // lowest slot j holding its own maximum, when that equals the warp's. (One ballot per
-    // slot and round before: ~1,200 warp instructions per token at 192 experts, top-8.)
-    unsigned key[TK];
+          for (int c = 0; c < 4; ++c)
 #pragma unroll
-    for (int j = 0; j < TK; ++j) {
-      const unsigned u = __float_as_uint(v[j] == 0.f ? 0.f : v[j]);
-      key[j] = (lane + 32 * j < E) ? ((u & 0x80000000u) ? ~u : (u | 0x80000000u)) : 0u;
-    }
-    float sel_v[8];
-    int sel_e[8];
+            for (int i = 0; i < 4; ++i) {
+              const int e = g0 + 4 * (c * LPT + q) + i;
+              if (e < E) z[c][i] = logits_in[size_t(t) * E + e];
+            }
+        } else {
+          const float *src = partial + size_t(t) * NE + g0 + 4 * q;
+          const size_t plane = size_t(T) * NE;
+          for (int y0 = 0; y0 < splits; y0 += 4) {  // summed in order
+            float4 v[4][4];
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      if (s >= k) break;
-      unsigned best = 0;
-      int bj = 0;
+            for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int j = 0; j < TK; ++j)
-        if (key[j] > best) {  // strict: the lowest slot keeps a tie
-          best = key[j];
-          bj = j;
+              for (int c = 0; c < 4; ++c)
+                if (y0 + u < splits && g0 + 4 * (c * LPT + q) < E)
+                  v[u][c] = *reinterpret_cast<const float4 *>(src + (y0 + u) * plane + 4 * LPT * c);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                if (y0 + u < splits && g0 + 4 * (c * LPT + q) < E) {
+                  z[c][0] += v[u][c].x;
+                  z[c][1] += v[u][c].y;
+                  z[c][2] += v[u][c].z;
+                  z[c][3] += v[u][c].w;
+                }
+          }
         }
-      const unsigned m = __reduce_max_sync(0xffffffffu, best);
-      const int be = int(__reduce_min_sync(0xffffffffu, best == m ? unsigned(32 * bj + lane) : ~0u));
+      }
 #pragma unroll
-      for (int j = 0; j < TK; ++j)
-        if (32 * j + lane == be) key[j] = 0u;
-      sel_v[s] = __uint_as_float((m & 0x80000000u) ? (m & 0x7fffffffu) : ~m);
-      sel_e[s] = be;
+      for (int c = 0; c < 4; ++c) {
+        const int e0 = g0 + 4 * (c * LPT + q);
+        if (e0 < E) {
+          if (logits_in == nullptr && bias != nullptr) {
+            const float4 b = *reinterpret_cast<const float4 *>(s_bias + e0);
+            z[c][0] += b.x;
+            z[c][1] += b.y;
+            z[c][2] += b.z;
+            z[c][3] += b.w;
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int e = e0 + i;
+            float v = z[c][i];
+            if (!s_live[e]) v = -INFINITY;
+            if (e < E) {
+              if (logits_out != nullptr && mine) logits_out[size_t(t) * E + e] = v;
+              // a larger float gives a larger key; -0 is taken as +0 so that equal logits tie
+              const unsigned u = __float_as_uint(v == 0.f ? 0.f : v);
+              top.add((u & 0x80000000u) ? ~u : (u | 0x80000000u), e);
+            }
+          }
+        }
+      }
     }
+    __syncwarp();
+#pragma unroll
+    for (int h = 1; h < LPT; h <<= 1) top.merge(h);
+    if (!mine) continue;
     // softmax over the selected logits (renormalised top-k), fp32
-    const float zmax = sel_v[0];
-    float den = 0.f, ex[8];
+    float ex[K], den = 0.f, zmax = 0.f;
     bool too_few = false;
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
+    for (int s = 0; s < K; ++s) {
       if (s < k) {
-        ex[s] = expf(sel_v[s] - zmax);
+        const unsigned m = top.key[s];
+        const float v = __uint_as_float((m & 0x80000000u) ? (m & 0x7fffffffu) : ~m);
+        if (s == 0) zmax = v;
+        ex[s] = expf(v - zmax);
         den += ex[s];
-        if (sel_v[s] == -INFINITY) too_few = true;
+        if (v == -INFINITY) too_few = true;
       }
     }
-    if (lane == 0 && too_few) dev_flag(&g_dev_err, MOE_DEV_TOO_FEW_LIVE);
+    if (q == 0 && too_few) dev_flag(&g_dev_err, MOE_DEV_TOO_FEW_LIVE);
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      if (s < k && lane == s) {
-        topk_idx[size_t(t) * k + s] = sel_e[s];
+    for (int s = 0; s < K; ++s) {
+      if (s < k && s % LPT == q) {
+        topk_idx[size_t(t) * k + s] = top.e[s];
         topk_gate[size_t(t) * k + s] = ex[s] / den;
-        if (sel_e[s] >= 0 && sel_e[s] < E) atomicAdd(&hist[sel_e[s]], 1);
+        if (top.e[s] >= 0) atomicAdd(&hist[top.e[s]], 1);
       }
     }
   }
   __syncthreads();
   if (counts != nullptr)
-    for (int e = tid; e < E; e += kRouteThreads)
+    for (int e = tid; e < E; e += kTopkThreads)
       if (hist[e]) atomicAdd(&counts[e], hist[e]);
 }
 
@@ -475,16 +627,35 @@ __global__ void route_bwd_dz_kernel(const int32_t *__restrict__ topk_idx,
   }
 }
 
-// dw_router[i, e] = sum over the splits, in order, of partial[split][i][e].
+// dw_router[i, e] = sum over the splits, in order, of partial[split][i][e]; four experts per thread,
+// four partials in flight.
 __global__ void route_dw_reduce_kernel(const float *__restrict__ partial, int splits, int d,
                                        int E, int NE, float *__restrict__ dw_router) {
   pdl_start();
-  const int n = d * E;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
-    const int i = idx / E, e = idx - i * E;
-    float acc = 0.f;
-    for (int y = 0; y < splits; ++y) acc += partial[(size_t(y) * d + i) * NE + e];
-    dw_router[idx] = acc;
+  const int n4 = NE / 4;
+  const size_t plane = size_t(d) * n4;
+  const float4 *src = reinterpret_cast<const float4 *>(partial);
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < d * n4; idx += gridDim.x * blockDim.x) {
+    const int i = idx / n4, e = 4 * (idx - i * n4);
+    if (e >= E) continue;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int y = 0; y < splits; y += 4) {
+      float4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (y + u < splits) v[u] = src[(y + u) * plane + idx];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (y + u < splits) {
+          acc[0] += v[u].x;
+          acc[1] += v[u].y;
+          acc[2] += v[u].z;
+          acc[3] += v[u].w;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (e + c < E) dw_router[size_t(i) * E + e + c] = acc[c];
   }
 }
 
@@ -493,20 +664,26 @@ __global__ void zero_f32_kernel(float *p, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0.f;
 }
 
+template <bool DW, int G>
+int launch_route_mma(const char *name, dim3 grid, size_t smem, const CUtensorMap &a, const CUtensorMap &b,
+                       const RouteTcParams &p, cudaStream_t s, const char *what) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(route_tc_kernel<DW, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRtMaxSmem);
+    if (e != cudaSuccess) return moe::cuda_status(e, what);
+    attr_set = true;
+  }
+  MOE_LAUNCH(name, s, moe::launch_dep(route_tc_kernel<DW, G>, grid, kRtThreads, smem, s, a, b, p));
+  return moe::launch_status(what);
+}
 // Tensor-core logits: splits W into its three bf16 terms (w3), then one CTA per
 // (token tile, split). Returns the number of partial planes written in *splits.
 int launch_route_tc(const uint16_t *x, const float *w, int T, int d, int E, int NE, uint16_t *w3,
                     float *partial, int32_t *counts, int *splits_out, cudaStream_t s) {
-  const int NP = route_tc_np(E), MT = route_tc_mt(NP);
-  const int stages = route_tc_stages(NP);
+  const int NP = route_tc_np(E);
+  const RtPlan plan = route_logits_plan(T, d, NP);
+  const int MT = plan.MT, stages = plan.stages, splits = plan.splits;
   const size_t smem = route_tc_smem(NP, stages, MT);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(route_tc_kernel<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kRtMaxSmem);
-    if (e != cudaSuccess) return moe::cuda_status(e, "moe_route: set smem attribute");
-    attr_set = true;
-  }
   dim3 sgrid((d + 31) / 32, (NP + 31) / 32);
   MOE_LAUNCH("route_split_w", s, moe::launch_dep(route_split_w_kernel, sgrid, dim3(32, 8), 0, s, w, d, E, NP, w3, counts));
   if (int st = moe::launch_status("moe_route: split router weight")) return st;
@@ -515,12 +692,10 @@ int launch_route_tc(const uint16_t *x, const float *w, int T, int d, int E, int 
   if ((st = moe::make_map(&mx, x, uint64_t(T), uint64_t(d), kRtBK, kRtBM, "router x"))) return st;
   if ((st = moe::make_map(&mw, w3, uint64_t(3 * NP), uint64_t(d), kRtBK, uint32_t(NP), "router w")))
     return st;
-  int splits = 1, per = 1;
-  route_tc_split(T, d, route_tc_np(E), &splits, &per);
   RouteTcParams p;
   p.M = T;
   p.MT = MT;
-  p.kb_per_split = per;
+  p.kb_per_split = plan.kb_per_split;
   p.nkb = (d + kRtBK - 1) / kRtBK;
   p.NP = NP;
   p.NE = NE;
@@ -528,26 +703,31 @@ int launch_route_tc(const uint16_t *x, const float *w, int T, int d, int E, int 
   p.tmem_cols = route_tc_tmem_cols(NP, MT);
   p.partial = partial;
   dim3 grid((T + kRtBM * MT - 1) / (kRtBM * MT), splits);
-  MOE_LAUNCH("route_logits", s, moe::launch_dep(route_tc_kernel<false>, grid, kRtThreads, smem, s, mx, mw, p));
   *splits_out = splits;
-  return moe::launch_status("moe_route: logits");
+  return launch_route_mma<false, 1>("route_logits", grid, smem, mx, mw, p, s, "moe_route: logits");
 }
 
-template <int NE>
 int launch_route(const uint16_t *x, const float *w, const float *b, const uint8_t *mask, int T,
                  int d, int E, int k, const float *lin, float *lout, int32_t *idx, float *gate,
                  int32_t *counts, float *partial, uint16_t *w3, cudaStream_t s) {
   int splits = 0;
+  const int NE = padded_experts(E);
   if (lin == nullptr)
     if (int st = launch_route_tc(x, w, T, d, E, NE, w3, partial, counts, &splits, s)) return st;
-  // one warp per token, grid-stride over the tokens; four blocks per SM, so that each
-  // block's shared histogram sums ~100 tokens' assignments before its global atomics (one
-  // block per 8 tokens sent 512k atomics to the counters at T=65536, top-8; the heaviest
-  // expert's counter took ~60k of them one after another)
-  const int grid2 = int(std::min<int64_t>((int64_t(T) + kRouteThreads / 32 - 1) / (kRouteThreads / 32),
-                                          int64_t(moe::num_sms()) * 4));
-  MOE_LAUNCH("route_topk", s, moe::launch_dep(route_topk_kernel<NE>, grid2, kRouteThreads, 0, s,
-                                  partial, splits, lin, b, mask, T, E, k, lout, idx, gate, counts));
+  // at most eight blocks per SM, so that each block's shared histogram sums ~50 tokens'
+  // assignments or more before its global atomics (one block per 8 tokens sent 512k atomics to
+  // the counters at T=65536, top-8; the heaviest expert's counter took ~60k of them one after
+  // another)
+  const bool wide = T <= 2048;  // 16 lanes per token: 6.5 against 16 us at T=764, 198 experts, 13 against 7 at T=8192, 64
+  const int per_block = kTopkThreads / (wide ? 16 : 4);
+  const int grid = int(std::min<int64_t>((int64_t(T) + per_block - 1) / per_block, int64_t(moe::num_sms()) * 8));
+  auto launch = [&](auto kern) {
+    MOE_LAUNCH("route_topk", s, moe::launch_dep(kern, grid, kTopkThreads, 0, s, partial, splits, NE, lin, b, mask, T, E,
+                                                k, lout, idx, gate, counts));
+  };
+  if (k <= 2) launch(wide ? route_topk_kernel<2, 16> : route_topk_kernel<2, 4>);
+  else if (k <= 4) launch(wide ? route_topk_kernel<4, 16> : route_topk_kernel<4, 4>);
+  else launch(wide ? route_topk_kernel<8, 16> : route_topk_kernel<8, 4>);
   return moe::launch_status("moe_route: top-k");
 }
 
@@ -558,8 +738,7 @@ MOE_DEV_ERR_DEFINE_READER(route_dev_error)
 
 size_t route_partial_bytes(int T, int d, int E) {
   if (T <= 0) return 0;
-  int splits = 1, per = 1;
-  route_tc_split(T, d, route_tc_np(E), &splits, &per);
+  const int splits = route_logits_plan(T, d, route_tc_np(E)).splits;
   return size_t(splits) * size_t(T) * size_t(padded_experts(E)) * 4;
 }
 size_t route_w3_bytes(int d, int E) { return size_t(3) * route_tc_np(E) * size_t(d) * 2; }
@@ -568,8 +747,7 @@ size_t route_dz3_bytes(int T, int E) {
 }
 size_t route_dw_partial_bytes(int T, int d, int E) {
   if (T <= 0) return 0;
-  int splits = 1, per = 1;
-  route_tc_split(d, route_tokens_padded(T), route_tc_np(E), &splits, &per);
+  const int splits = route_dw_plan(d, route_tokens_padded(T), route_tc_np(E)).splits;
   return size_t(splits) * size_t(d) * size_t(route_dw_stride(E)) * 4;
 }
 }  // namespace moe
@@ -602,12 +780,8 @@ int moe_route(const uint16_t *x, const float *w_router, const float *bias,
     if (int st = moe::launch_status("moe_route: zero counts")) return st;
   }
   if (T == 0) return MOE_OK;
-  switch (padded_experts(E)) {
-    case 64: return launch_route<64>(x, w_router, bias, active_mask, T, d, E, k, logits_in, logits_out, topk_idx, topk_gate, counts, partial, w3, s);
-    case 128: return launch_route<128>(x, w_router, bias, active_mask, T, d, E, k, logits_in, logits_out, topk_idx, topk_gate, counts, partial, w3, s);
-    case 192: return launch_route<192>(x, w_router, bias, active_mask, T, d, E, k, logits_in, logits_out, topk_idx, topk_gate, counts, partial, w3, s);
-    default: return launch_route<256>(x, w_router, bias, active_mask, T, d, E, k, logits_in, logits_out, topk_idx, topk_gate, counts, partial, w3, s);
-  }
+  return launch_route(x, w_router, bias, active_mask, T, d, E, k, logits_in, logits_out, topk_idx, topk_gate, counts,
+                      partial, w3, s);
 }
 
 int moe_load_stats(const int32_t *topk_idx, int T, int k, int E, int32_t *counts, int accumulate,
@@ -632,38 +806,34 @@ namespace {
 // Weight-gradient launch on the tensor cores: partial[split][i][e] over the split's tokens.
 int launch_route_dw(const uint16_t *x, const uint16_t *dz3, int T, int d, int E, float *partial,
                     int *splits_out, cudaStream_t s) {
-  const int NP = route_tc_np(E), Tp = route_tokens_padded(T), MT = route_tc_mt(NP);
-  const int stages = route_tc_stages(NP);
+  const int NP = route_tc_np(E), Tp = route_tokens_padded(T);
+  const RtPlan plan = route_dw_plan(d, Tp, NP);
+  const int MT = plan.MT, stages = plan.stages, splits = plan.splits;
   const size_t smem = route_tc_smem(NP, stages, MT);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(route_tc_kernel<true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kRtMaxSmem);
-    if (e != cudaSuccess) return moe::cuda_status(e, "moe_route_bwd: set smem attribute");
-    attr_set = true;
-  }
   CUtensorMap mx, mz;
   int st;
   // x [T, d] read as 64 features x 64 tokens boxes (features contiguous: MN-major A)
   if ((st = moe::make_map(&mx, x, uint64_t(T), uint64_t(d), 64, kRtBK, "router bwd x"))) return st;
   if ((st = moe::make_map(&mz, dz3, uint64_t(3 * NP), uint64_t(Tp), kRtBK, uint32_t(NP), "router bwd dz")))
     return st;
-  int splits = 1, per = 1;
-  route_tc_split(d, Tp, NP, &splits, &per);
   RouteTcParams p;
   p.M = d;
   p.MT = MT;
-  p.kb_per_split = per;
+  p.kb_per_split = plan.kb_per_split;
   p.nkb = Tp / kRtBK;
   p.NP = NP;
   p.NE = route_dw_stride(E);
   p.stages = stages;
-  p.tmem_cols = route_tc_tmem_cols(NP, MT);
+  p.tmem_cols = route_tc_tmem_cols(route_dw_group(NP) * NP, MT);
   p.partial = partial;
   dim3 grid((d + kRtBM * MT - 1) / (kRtBM * MT), splits);
-  MOE_LAUNCH("route_bwd_dw", s, moe::launch_dep(route_tc_kernel<true>, grid, kRtThreads, smem, s, mx, mz, p));
   *splits_out = splits;
-  return moe::launch_status("moe_route_bwd: weight gradient");
+  const char *what = "moe_route_bwd: weight gradient";
+  switch (route_dw_group(NP)) {
+    case 1: return launch_route_mma<true, 1>("route_bwd_dw", grid, smem, mx, mz, p, s, what);
+    case 2: return launch_route_mma<true, 2>("route_bwd_dw", grid, smem, mx, mz, p, s, what);
+    default: return launch_route_mma<true, 3>("route_bwd_dw", grid, smem, mx, mz, p, s, what);
+  }
 }
 }  // namespace
 
@@ -695,7 +865,7 @@ int moe_route_bwd(const uint16_t *x, const int32_t *topk_idx, const float *topk_
   if (int st = moe::launch_status("moe_route_bwd: dz")) return st;
   int splits = 0;
   if (int st = launch_route_dw(x, dz3, T, d, E, partial, &splits, s)) return st;
-  const int n = d * E;
+  const int n = d * (route_dw_stride(E) / 4);
   MOE_LAUNCH("route_bwd_reduce", s, moe::launch_dep(route_dw_reduce_kernel, std::min((n + 255) / 256, 4 * moe::num_sms()), 256, 0, s,
                                         partial, splits, d, E, route_dw_stride(E), dw_router));
   return moe::launch_status("moe_route_bwd: reduce");

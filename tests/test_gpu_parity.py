@@ -75,7 +75,10 @@ def test_route_ties_go_to_lower_index():
                                    (1000, 384, 100), (2500, 7168, 171),
                                    # d not a multiple of the 64-wide k-block (zero-filled tail),
                                    # few experts (MMA N = 16), one token, the smallest d
-                                   (333, 200, 13), (1, 72, 256), (64, 8, 5), (50, 136, 2)])
+                                   (333, 200, 13), (1, 72, 256), (64, 8, 5), (50, 136, 2),
+                                   # three, two and one weight terms per MMA at the edges of each
+                                   # (80 / 81, 128 / 129 experts), many splits, two tiles per CTA
+                                   (40, 4096, 80), (5000, 1000, 81), (20000, 264, 128), (257, 2048, 129)])
 def test_route_logits_fp32(T, d, E):
     inp = case_inputs(T, d, E, 2, 128, seed=5)
     o = oracle_inputs(inp)
@@ -101,7 +104,9 @@ def test_route_logits_fp32(T, d, E):
                                      # tokens not a multiple of the 64-token k-block, d not a
                                      # multiple of the 128-feature tile, MMA N = 16, one token
                                      (333, 136, 13, 2), (1, 72, 5, 1), (64, 8, 2, 2),
-                                     (4100, 1024, 16, 2)])
+                                     (4100, 1024, 16, 2),
+                                     # many splits, experts at the edges of the terms per MMA
+                                     (9000, 136, 80, 3), (6000, 264, 81, 8), (5000, 1032, 129, 2)])
 def test_route_bwd_against_oracle(T, d, E, k):
     """moe_route_bwd alone, from the same fp32 gates and d_gate as the oracle."""
     dev = "cuda"
@@ -134,6 +139,28 @@ def test_route_bwd_against_oracle(T, d, E, k):
     assert (np.abs(got - dw_ref) <= 1e-5 * scale + 1e-30).all()
     unused = np.setdiff1d(np.arange(E), idx.numpy())
     assert (got[:, unused] == 0).all()
+
+
+@pytest.mark.parametrize("T,E,k,n_masked", [(2048, 16, 1, 0), (2049, 17, 2, 3), (300, 256, 3, 100),
+                                            (3000, 255, 4, 0), (77, 64, 5, 59), (2500, 65, 8, 1),
+                                            (1, 8, 8, 0), (5000, 130, 7, 120), (9, 1, 1, 0)])
+def test_route_topk_ties_bit_exact(T, E, k, n_masked):
+    """Every list length and lane count of the top-k (16 lanes per token up to 2048 tokens, then
+    4), logits with many exact ties, infinities and both zeros, masked experts: ties to the lower
+    index, bit for bit."""
+    rng = np.random.default_rng(T + E)
+    z = rng.integers(-3, 3, size=(T, E)).astype(np.float32)
+    z[(z == 0) & (rng.random(z.shape) < 0.5)] = -0.0
+    z[rng.random(z.shape) < 0.02] = np.finfo(np.float32).min
+    mask = np.ones(E, np.uint8)
+    mask[rng.permutation(E)[:n_masked]] = 0
+    idx, g, cnt, lo = _route_only(T, E, k, z, mask)
+    zm = O.apply_mask(z, mask)
+    oidx, og = O.route_topk(zm, k)
+    assert (idx == oidx).all()
+    np.testing.assert_allclose(g, og, rtol=0, atol=2e-6)
+    assert (cnt == O.expert_counts(oidx, E)).all()
+    assert (lo == zm).all()
 
 
 def test_load_stats_bit_exact_and_accumulate():
