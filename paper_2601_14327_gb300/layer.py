@@ -102,6 +102,7 @@ def forward(b: MoELayerBuffers, x, w_router, bias, w_gate_up, w_down, active_mas
     when b.fused_combine). Returns b.y."""
     s = b.shape
     R = s.rows_cap
+    stream = L.stream_handle(stream)  # once for all calls
     route(b, x, w_router, bias, active_mask, logits_in, keep_logits, stream)
     b.x = x
     if b.gather:
@@ -145,8 +146,11 @@ def backward(b: MoELayerBuffers, dy, w_router, w_gate_up, w_down, stream=None,
     Returns (dx, dw_gate_up, dw_down, dw_router)."""
     s = b.shape
     R = s.rows_cap
-    main = torch.cuda.current_stream() if stream is None else stream
-    side = b.side if overlap else main
+    if overlap:
+        main = torch.cuda.current_stream() if stream is None else stream
+        side = b.side
+    else:
+        main = side = L.stream_handle(stream)  # once for all calls
     # d_out_perm = g * dy; the gate gradient comes from the dH GEMM (below), so the combine
     # backward does not read out_perm
     L.moe_unpermute_combine_bwd(dy, None, b.row_of_assignment, b.topk_gate,
