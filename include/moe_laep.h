@@ -271,7 +271,8 @@ int moe_permute_noalloc(const uint16_t *x, const int32_t *topk_idx, const int32_
  * 76th one (with rows_cap >= 2^18, a group's odd last 128-row block is computed
  * by a second, one-SM launch on the same stream). With few rows per expert (up to
  * 640 on average, fewer for long reductions) those GEMMs run on single SMs, in
- * 128-row tiles. A tile's arithmetic depends neither on which pair or SM runs it nor
+ * 128-row tiles; so do the weight gradients up to 128 rows (or short tile lists), each
+ * SM taking every 152nd tile of the list. A tile's arithmetic depends neither on which pair or SM runs it nor
  * on the tiles' shape: results are bitwise reproducible.
  * Limits: d % 128 == 0, F % 128 == 0, all pointers 16-byte aligned.
  */

@@ -21,6 +21,7 @@ SCHEDULE_CASES = [
     (1500, 384, 12, 4, 640, "loguniform"),
     (3000, 256, 256, 8, 256, "zipf"),
     (8192, 512, 64, 6, 512, "zipf"),
+    (3000, 512, 64, 8, 512, "zipf"),  # CTA pairs with many light experts: claims of several tiles
 ]
 NAMES = ["y", "dx", "h", "out_perm", "d_ab", "dx_perm", "dw_gate_up", "dw_down", "dw_router"]
 GROUPED = {"h", "out_perm", "d_ab", "dx_perm"}  # rows past group_offsets[E] are never written
