@@ -194,36 +194,46 @@ __device__ __forceinline__ void zero_pad_rows(int b, const int32_t *__restrict__
     for (int c = threadIdx.x & 31; c < nv; c += 32) stg_v4(buf + size_t(r) * d + c * 8, z);
 }
 
-// One warp per token: read x[t,:] once, write it to its k grouped rows. Blocks below
+// Token and column segment of a warp: nseg warps share a token, warp `seg` taking its 16-byte
+// vectors lane + 32 (seg + nseg i) (see token_segments). False past the last token.
+__device__ __forceinline__ bool token_segment(int block, int T, int nseg, int *t, int *seg) {
+  const int w = block * kWarps + int(threadIdx.x >> 5);
+  *t = w / nseg;
+  *seg = w - *t * nseg;
+  return *t < T;
+}
+
+// One warp (or nseg) per token: read x[t,:] once, write it to its k grouped rows. Blocks below
 // pad_blocks zero padding rows.
+// (SEG: nseg > 1; the fixed strides of the other form are worth 2% at T=16384.)
+template <bool SEG>
 __global__ void __launch_bounds__(kThreads) perm_gather_kernel(
     const uint16_t *__restrict__ x, const int32_t *__restrict__ row_of_assignment, int T, int d,
-    int k, int64_t rows_cap, int pad_blocks, const int32_t *__restrict__ group_offsets,
+    int k, int nseg, int64_t rows_cap, int pad_blocks, const int32_t *__restrict__ group_offsets,
     const int32_t *__restrict__ group_counts, uint16_t *__restrict__ x_perm) {
   pdl_start();
   if (int(blockIdx.x) < pad_blocks) {
     zero_pad_rows(blockIdx.x, group_offsets, group_counts, d, rows_cap, x_perm);
     return;
   }
-  const int warp = ((blockIdx.x - pad_blocks) * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (warp >= T) return;
-  const int t = warp;
+  int t, seg;
+  if (!token_segment(blockIdx.x - pad_blocks, T, SEG ? nseg : 1, &t, &seg)) return;
   int my_row = (lane < k) ? row_of_assignment[size_t(t) * k + lane] : -1;
   int rows[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) rows[j] = __shfl_sync(0xffffffffu, my_row, j);
-  const int nv = d / 8;
+  const int nv = d / 8, step = SEG ? 32 * nseg : 32;
   const uint16_t *src = x + size_t(t) * d;
   // four 16-byte loads in flight per lane before their stores
-  for (int c0 = lane; c0 < nv; c0 += 128) {
+  for (int c0 = lane + 32 * seg; c0 < nv; c0 += 4 * step) {
     uint4 v[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      if (c0 + 32 * u < nv) v[u] = ldg_nc_v4(src + (c0 + 32 * u) * 8);
+      if (c0 + step * u < nv) v[u] = ldg_nc_v4(src + (c0 + step * u) * 8);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int c = c0 + 32 * u;
+      const int c = c0 + step * u;
       if (c >= nv) break;
 #pragma unroll
       for (int j = 0; j < 8; ++j)
@@ -235,12 +245,11 @@ __global__ void __launch_bounds__(kThreads) perm_gather_kernel(
 // y[t] = sum_j g[t,j] * out_perm[row(t,j)]  (fp32 sum, one bf16 rounding)
 __global__ void __launch_bounds__(kThreads) combine_kernel(
     const uint16_t *__restrict__ out_perm, const int32_t *__restrict__ row_of_assignment,
-    const float *__restrict__ gate, int T, int d, int k, uint16_t *__restrict__ y) {
+    const float *__restrict__ gate, int T, int d, int k, int nseg, uint16_t *__restrict__ y) {
   pdl_start();
-  const int warp = (blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (warp >= T) return;
-  const int t = warp;
+  int t, seg;
+  if (!token_segment(blockIdx.x, T, nseg, &t, &seg)) return;
   int my_row = (lane < k) ? row_of_assignment[size_t(t) * k + lane] : -1;
   float my_g = (lane < k) ? gate[size_t(t) * k + lane] : 0.f;
   int rows[8];
@@ -251,7 +260,7 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(
     g[j] = __shfl_sync(0xffffffffu, my_g, j);
   }
   const int nv = d / 8;
-  for (int c = lane; c < nv; c += 32) {
+  for (int c = lane + 32 * seg; c < nv; c += 32 * nseg) {
     uint4 v[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j)
@@ -274,12 +283,12 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(
 // DOUT: d_out_perm rows = g * dy[t]; DGATE: d_gate = <dy[t], out_perm rows>. The two
 // halves can run as separate launches (DGATE alone reads out_perm and writes nothing
 // large; DOUT alone never reads out_perm). Blocks below pad_blocks (DOUT only) zero
-// padding rows of d_out_perm.
+// padding rows of d_out_perm. nseg is 1 with DGATE, whose sums run over the whole row.
 template <bool DOUT, bool DGATE>
 __global__ void __launch_bounds__(kThreads) combine_bwd_kernel(
     const uint16_t *__restrict__ dy, const uint16_t *__restrict__ out_perm,
     const int32_t *__restrict__ row_of_assignment, const float *__restrict__ gate, int T, int d,
-    int k, int64_t rows_cap, int pad_blocks, const int32_t *__restrict__ group_offsets,
+    int k, int nseg, int64_t rows_cap, int pad_blocks, const int32_t *__restrict__ group_offsets,
     const int32_t *__restrict__ group_counts, uint16_t *__restrict__ d_out_perm,
     float *__restrict__ d_gate) {
   pdl_start();
@@ -287,10 +296,9 @@ __global__ void __launch_bounds__(kThreads) combine_bwd_kernel(
     zero_pad_rows(blockIdx.x, group_offsets, group_counts, d, rows_cap, d_out_perm);
     return;
   }
-  const int warp = ((blockIdx.x - pad_blocks) * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (warp >= T) return;
-  const int t = warp;
+  int t, seg;
+  if (!token_segment(blockIdx.x - pad_blocks, T, nseg, &t, &seg)) return;
   int my_row = (lane < k) ? row_of_assignment[size_t(t) * k + lane] : -1;
   float my_g = (lane < k) ? gate[size_t(t) * k + lane] : 0.f;
   int rows[8];
@@ -303,7 +311,7 @@ __global__ void __launch_bounds__(kThreads) combine_bwd_kernel(
     dot[j] = 0.f;
   }
   const int nv = d / 8;
-  for (int c = lane; c < nv; c += 32) {
+  for (int c = lane + 32 * seg; c < nv; c += 32 * nseg) {
     float fd[8];
     unpack8(ldg_nc_v4(dy + size_t(t) * d + c * 8), fd);
     uint4 v[8];
@@ -362,12 +370,11 @@ __global__ void transpose_router_kernel(const float *__restrict__ w, int d, int 
 __global__ void __launch_bounds__(kThreads) permute_bwd_kernel(
     const uint16_t *__restrict__ dx_perm, const int32_t *__restrict__ row_of_assignment,
     const int32_t *__restrict__ topk_idx, const float *__restrict__ d_logits,
-    const float *__restrict__ w_t, int T, int d, int E, int k, uint16_t *__restrict__ dx) {
+    const float *__restrict__ w_t, int T, int d, int E, int k, int nseg, uint16_t *__restrict__ dx) {
   pdl_start();
-  const int warp = (blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (warp >= T) return;
-  const int t = warp;
+  int t, seg;
+  if (!token_segment(blockIdx.x, T, nseg, &t, &seg)) return;
   const bool router = (d_logits != nullptr && w_t != nullptr);
   int my_row = (lane < k) ? row_of_assignment[size_t(t) * k + lane] : -1;
   int my_e = (lane < k && router) ? topk_idx[size_t(t) * k + lane] : -1;
@@ -382,7 +389,7 @@ __global__ void __launch_bounds__(kThreads) permute_bwd_kernel(
     dz[j] = __shfl_sync(0xffffffffu, my_dz, j);
   }
   const int nv = d / 8;
-  for (int c = lane; c < nv; c += 32) {
+  for (int c = lane + 32 * seg; c < nv; c += 32 * nseg) {
     uint4 v[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j)
@@ -414,7 +421,18 @@ __global__ void __launch_bounds__(kThreads) permute_bwd_kernel(
   }
 }
 
-int warp_grid(int T) { return (T + kWarps - 1) / kWarps; }
+// Warps per token of the row kernels: one from `per_sm` warps per SM on, and with fewer tokens as
+// many as give that, up to one per 32 of the row's 16-byte vectors. A lone warp's row is a chain
+// of d / 256 loads' latencies: combine over 37 tokens (d 2048, top-6) 5.2 -> 2.0 us, over 191
+// (d 7064, top-8) 16.2 -> 4.0 us; from ~1,000 tokens on the warps of other tokens hide it. The
+// gather writes k rows per load and loses by shorter pieces sooner (T=100, d 7168: 26.8 -> 17.9
+// us; T=800, d 4096: 20.9 -> 22.9 us).
+constexpr int kCombineWarpsPerSm = 8, kGatherWarpsPerSm = 4;
+int token_segments(int T, int d, int per_sm) {
+  const int64_t warps = int64_t(moe::num_sms()) * per_sm, most = (d / 8 + 31) / 32;
+  return int(std::max<int64_t>(1, std::min(most, warps / std::max(T, 1))));
+}
+int token_grid(int T, int nseg) { return int((int64_t(T) * nseg + kWarps - 1) / kWarps); }
 
 // The grouped layout: group_offsets, group_counts, row_of_assignment (and token_of_row when
 // given). One chunk of assignments is one launch; more take the block histograms first.
@@ -435,9 +453,10 @@ int launch_layout(const int32_t *idx, int64_t A, int E, int32_t *hist, const int
 int launch_gather(const uint16_t *x, const int32_t *row, int T, int d, int E, int k, int64_t rows_cap,
                   const int32_t *group_offsets, const int32_t *group_counts, uint16_t *x_perm,
                   cudaStream_t s, const char *what) {
-  const int pad = E * kPadSplit;
-  MOE_LAUNCH("perm_gather", s, moe::launch_dep(perm_gather_kernel, pad + warp_grid(T), kThreads, 0, s, x, row, T, d, k,
-                                               rows_cap, pad, group_offsets, group_counts, x_perm));
+  const int pad = E * kPadSplit, nseg = token_segments(T, d, kGatherWarpsPerSm);
+  auto kern = nseg > 1 ? perm_gather_kernel<true> : perm_gather_kernel<false>;
+  MOE_LAUNCH("perm_gather", s, moe::launch_dep(kern, pad + token_grid(T, nseg), kThreads, 0, s, x, row, T, d, k,
+                                               nseg, rows_cap, pad, group_offsets, group_counts, x_perm));
   return moe::launch_status(what);
 }
 
@@ -510,7 +529,8 @@ int moe_unpermute_combine(const uint16_t *out_perm, const int32_t *row_of_assign
     return moe::set_error(MOE_ERR_ARG, "moe_unpermute_combine: null pointer");
   if (!moe::aligned16(out_perm) || !moe::aligned16(y))
     return moe::set_error(MOE_ERR_ARG, "moe_unpermute_combine: alignment");
-  MOE_LAUNCH("combine", s, moe::launch_dep(combine_kernel, warp_grid(T), kThreads, 0, s, out_perm, row_of_assignment, topk_gate, T, d, k, y));
+  const int nseg = token_segments(T, d, kCombineWarpsPerSm);
+  MOE_LAUNCH("combine", s, moe::launch_dep(combine_kernel, token_grid(T, nseg), kThreads, 0, s, out_perm, row_of_assignment, topk_gate, T, d, k, nseg, y));
   return moe::launch_status("moe_unpermute_combine: launch");
 }
 
@@ -532,18 +552,19 @@ int moe_unpermute_combine_bwd(const uint16_t *dy, const uint16_t *out_perm,
     return moe::set_error(MOE_ERR_ARG, "moe_unpermute_combine_bwd: alignment");
   const int64_t rows_cap = moe_perm_rows_max(T, k, E);
   if (T == 0 && !d_out_perm) return MOE_OK;
-  const int pad = d_out_perm ? E * kPadSplit : 0, grid = pad + warp_grid(T);
+  const int nseg = d_gate ? 1 : token_segments(T, d, kCombineWarpsPerSm);
+  const int pad = d_out_perm ? E * kPadSplit : 0, grid = pad + token_grid(T, nseg);
   if (d_out_perm && d_gate) {
     MOE_LAUNCH("combine_bwd", s, moe::launch_dep(combine_bwd_kernel<true, true>, grid, kThreads, 0, s, dy, out_perm,
-                                                 row_of_assignment, topk_gate, T, d, k, rows_cap, pad,
+                                                 row_of_assignment, topk_gate, T, d, k, nseg, rows_cap, pad,
                                                  group_offsets, group_counts, d_out_perm, d_gate));
   } else if (d_out_perm) {
     MOE_LAUNCH("combine_bwd_dout", s, moe::launch_dep(combine_bwd_kernel<true, false>, grid, kThreads, 0, s, dy,
-                                                      out_perm, row_of_assignment, topk_gate, T, d, k, rows_cap,
+                                                      out_perm, row_of_assignment, topk_gate, T, d, k, nseg, rows_cap,
                                                       pad, group_offsets, group_counts, d_out_perm, d_gate));
   } else {
     MOE_LAUNCH("combine_bwd_dgate", s, moe::launch_dep(combine_bwd_kernel<false, true>, grid, kThreads, 0, s, dy,
-                                                       out_perm, row_of_assignment, topk_gate, T, d, k, rows_cap,
+                                                       out_perm, row_of_assignment, topk_gate, T, d, k, nseg, rows_cap,
                                                        pad, group_offsets, group_counts, d_out_perm, d_gate));
   }
   return moe::launch_status("moe_unpermute_combine_bwd: launch");
@@ -572,8 +593,9 @@ int moe_permute_bwd(const uint16_t *dx_perm, const int32_t *row_of_assignment,
     MOE_LAUNCH("transpose_router", s, moe::launch_dep(transpose_router_kernel, grid, block, 0, s, w_router, d, E, w_t));
     if (int st = moe::launch_status("moe_permute_bwd: transpose")) return st;
   }
-  MOE_LAUNCH("permute_bwd", s, moe::launch_dep(permute_bwd_kernel, warp_grid(T), kThreads, 0, s, dx_perm,
-                                               row_of_assignment, topk_idx, d_logits, w_t, T, d, E, k, dx));
+  const int nseg = token_segments(T, d, kCombineWarpsPerSm);
+  MOE_LAUNCH("permute_bwd", s, moe::launch_dep(permute_bwd_kernel, token_grid(T, nseg), kThreads, 0, s, dx_perm,
+                                               row_of_assignment, topk_idx, d_logits, w_t, T, d, E, k, nseg, dx));
   return moe::launch_status("moe_permute_bwd: launch");
 }
 

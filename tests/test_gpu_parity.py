@@ -699,6 +699,42 @@ def test_combine_bwd_halves_equal_fused():
         L.moe_unpermute_combine_bwd(*args, None, None)
 
 
+@pytest.mark.parametrize("T,d,k", [(1, 8, 1), (1, 7168, 8), (37, 2048, 6), (151, 264, 3), (608, 520, 2),
+                                   (1217, 1032, 4)])
+def test_row_kernels_with_few_tokens(T, d, k):
+    """Gather, combine, combine backward and unpermute-sum where several warps share a token's
+    row (few tokens), one warp past a row's last vectors, and one warp per token, against fp32
+    sums in the same order. Bound: one bf16 rounding (2^-8) and the k fp32 additions."""
+    E, dev = 9, "cuda"
+    gen = torch.Generator(device=dev).manual_seed(T + d)
+    idx = torch.argsort(torch.rand(T, E, generator=gen, device=dev), dim=1)[:, :k].to(torch.int32).contiguous()
+    gate = torch.rand(T, k, generator=gen, device=dev)
+    x = torch.randn(T, d, generator=gen, device=dev).to(torch.bfloat16)
+    R = L.moe_perm_rows_max(T, k, E)
+    nb = max(L.moe_workspace_size(T, d, E, k, 128), 256)
+    ws = torch.empty(nb, dtype=torch.uint8, device=dev)
+    off, cnt = (torch.empty(n, dtype=torch.int32, device=dev) for n in (E + 1, E))
+    row = torch.empty(T, k, dtype=torch.int32, device=dev)
+    nan = lambda *s: torch.full(s, float("nan"), dtype=torch.bfloat16, device=dev)
+    xp, dop, y, dx = nan(R, d), nan(R, d), nan(T, d), nan(T, d)
+    L.moe_permute(x, idx, None, T, d, E, k, R, off, cnt, row, xp, ws, nb)
+    L.moe_unpermute_combine_bwd(x, None, row, gate, off, cnt, T, d, E, k, dop, None)
+    rows, used = row.reshape(-1).long(), int(off[-1])
+    want = torch.zeros(used, d, dtype=torch.bfloat16, device=dev)
+    want[rows] = x.repeat_interleave(k, dim=0)
+    assert torch.equal(xp[:used], want)
+    want = torch.zeros(used, d, dtype=torch.bfloat16, device=dev)
+    want[rows] = (gate.reshape(-1, 1) * x.float().repeat_interleave(k, dim=0)).to(torch.bfloat16)
+    assert torch.equal(dop[:used], want)
+    o = torch.randn(R, d, generator=gen, device=dev).to(torch.bfloat16)
+    L.moe_unpermute_combine(o, row, gate, T, d, k, y)
+    L.moe_permute_bwd(o, row, idx, None, None, T, d, E, k, dx, ws, nb)
+    og = o[rows].double().reshape(T, k, d)
+    for got, terms in ((y, gate.double()[:, :, None] * og), (dx, og)):
+        ref = terms.sum(1)
+        assert ((got.double() - ref).abs() <= 2.0**-8 * ref.abs() + k * 2.0**-23 * terms.abs().sum(1)).all()
+
+
 def test_layer_is_deterministic_and_stream_layout_independent():
     """Every reduction runs in a fixed order (split partials, router partial sums, combine
     sums) and the only atomics are integer counts, so a step gives the same bits every
