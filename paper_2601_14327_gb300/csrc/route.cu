@@ -555,7 +555,8 @@ __global__ void __launch_bounds__(kTopkThreads) route_topk_kernel(
       if (hist[e]) atomicAdd(&counts[e], hist[e]);
 }
 
-__global__ void load_stats_kernel(const int32_t *__restrict__ topk_idx, int64_t A, int E,
+// store: the only block of the launch, which writes the counts instead of adding to them.
+__global__ void load_stats_kernel(const int32_t *__restrict__ topk_idx, int64_t A, int E, int store,
                                   int32_t *__restrict__ counts) {
   __shared__ int hist[256];
   for (int e = threadIdx.x; e < E; e += blockDim.x) hist[e] = 0;
@@ -570,8 +571,10 @@ __global__ void load_stats_kernel(const int32_t *__restrict__ topk_idx, int64_t 
       dev_flag(&g_dev_err, MOE_DEV_BAD_EXPERT);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < E; e += blockDim.x)
-    if (hist[e]) atomicAdd(&counts[e], hist[e]);
+  for (int e = threadIdx.x; e < E; e += blockDim.x) {
+    if (store) counts[e] = hist[e];
+    else if (hist[e]) atomicAdd(&counts[e], hist[e]);
+  }
 }
 
 // ---- router backward -------------------------------------------------------
@@ -789,14 +792,18 @@ int moe_load_stats(const int32_t *topk_idx, int T, int k, int E, int32_t *counts
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (E < 1 || E > 256 || k < 1 || T < 0) return moe::set_error(MOE_ERR_ARG, "moe_load_stats: sizes");
   if (!counts || (T > 0 && !topk_idx)) return moe::set_error(MOE_ERR_ARG, "moe_load_stats: null");
+  const int64_t A = int64_t(T) * k;
+  if (!accumulate && A <= 8192) {  // one block (8 loads per thread), no launch to zero the counts
+    MOE_LAUNCH("load_stats", s, moe::launch_dep(load_stats_kernel, 1, 1024, 0, s, topk_idx, A, E, 1, counts));
+    return moe::launch_status("moe_load_stats: launch");
+  }
   if (!accumulate) {
     MOE_LAUNCH("zero_counts", s, moe::launch_dep(zero_i32_kernel, 1, 256, 0, s, counts, E));
     if (int st = moe::launch_status("moe_load_stats: zero")) return st;
   }
-  const int64_t A = int64_t(T) * k;
   if (A == 0) return MOE_OK;
   const int grid = int(std::min<int64_t>((A + 255) / 256, int64_t(moe::num_sms()) * 4));
-  MOE_LAUNCH("load_stats", s, moe::launch_dep(load_stats_kernel, grid, 256, 0, s, topk_idx, A, E, counts));
+  MOE_LAUNCH("load_stats", s, moe::launch_dep(load_stats_kernel, grid, 256, 0, s, topk_idx, A, E, 0, counts));
   return moe::launch_status("moe_load_stats: launch");
 }
 

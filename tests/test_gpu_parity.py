@@ -175,6 +175,17 @@ def test_load_stats_bit_exact_and_accumulate():
     assert (cnt.cpu().numpy() == 2 * np.bincount(idx.reshape(-1), minlength=E)).all()
 
 
+@pytest.mark.parametrize("T,k", [(0, 8), (1, 1), (1024, 8), (8193, 1)])  # one block up to 8192 assignments
+def test_load_stats_overwrites(T, k):
+    E = 77
+    idx = np.random.default_rng(T).integers(0, E, size=(T, k)).astype(np.int32)
+    cnt = torch.full((E,), -5, dtype=torch.int32, device="cuda")
+    L.moe_load_stats(torch.from_numpy(idx).cuda(), T, k, E, cnt)
+    assert (cnt.cpu().numpy() == np.bincount(idx.reshape(-1), minlength=E)).all()
+    L.moe_load_stats(torch.from_numpy(idx).cuda(), T, k, E, cnt, accumulate=True)
+    assert (cnt.cpu().numpy() == 2 * np.bincount(idx.reshape(-1), minlength=E)).all()
+
+
 def test_load_stats_flags_bad_expert():
     idx = torch.tensor([[0, 1], [2, 9]], dtype=torch.int32, device="cuda")
     cnt = torch.empty(4, dtype=torch.int32, device="cuda")
