@@ -193,7 +193,8 @@ __global__ void route_split_w_kernel(const float *__restrict__ w, int d, int E, 
 // boxes per k-block; B = dZ's three bf16 terms, K-major [3][NP][T padded to 64]).
 // G = terms per MMA (see route_dw_group), at compile time: the issuing thread's loop sets the pace
 // otherwise (with a bound read from the parameters 110 instead of 79 us at T=32768, 128 experts).
-template <bool DW, int G>
+// AHEAD (logits): a stage's next x tile goes to L2 while this one loads (see launch_route_tc).
+template <bool DW, int G, bool AHEAD>
 __global__ void __launch_bounds__(kRtThreads, 1)
     route_tc_kernel(const __grid_constant__ CUtensorMap tmX,
                     const __grid_constant__ CUtensorMap tmW, const RouteTcParams p) {
@@ -276,6 +277,13 @@ __global__ void __launch_bounds__(kRtThreads, 1)
 #pragma unroll
       for (int j = 0; j < 3; ++j)
         tc::tma_load_2d(dst + a_bytes + j * b_bytes, &tmW, full_bar(s), k0, j * p.NP);
+      if (AHEAD && int(it) + 2 < nk) {
+        const int k2 = (kb0 + (int(it) + 2 + rot) % nk) * kRtBK;
+        for (int m = 0; m < p.MT; ++m) {
+          const int row0 = (mt * p.MT + m) * kRtBM;
+          if (row0 < p.M) tc::tma_prefetch_2d(&tmX, k2, row0);
+        }
+      }
     }
     // every issued load lands before the CTA may exit (also after an abort)
     for (int s = 0; s < S; ++s) {
@@ -667,16 +675,16 @@ __global__ void zero_f32_kernel(float *p, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0.f;
 }
 
-template <bool DW, int G>
+template <bool DW, int G, bool AHEAD = false>
 int launch_route_mma(const char *name, dim3 grid, size_t smem, const CUtensorMap &a, const CUtensorMap &b,
                        const RouteTcParams &p, cudaStream_t s, const char *what) {
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(route_tc_kernel<DW, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRtMaxSmem);
+    cudaError_t e = cudaFuncSetAttribute(route_tc_kernel<DW, G, AHEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRtMaxSmem);
     if (e != cudaSuccess) return moe::cuda_status(e, what);
     attr_set = true;
   }
-  MOE_LAUNCH(name, s, moe::launch_dep(route_tc_kernel<DW, G>, grid, kRtThreads, smem, s, a, b, p));
+  MOE_LAUNCH(name, s, moe::launch_dep(route_tc_kernel<DW, G, AHEAD>, grid, kRtThreads, smem, s, a, b, p));
   return moe::launch_status(what);
 }
 // Tensor-core logits: splits W into its three bf16 terms (w3), then one CTA per
@@ -707,7 +715,19 @@ int launch_route_tc(const uint16_t *x, const float *w, int T, int d, int E, int 
   p.partial = partial;
   dim3 grid((T + kRtBM * MT - 1) / (kRtBM * MT), splits);
   *splits_out = splits;
-  return launch_route_mma<false, 1>("route_logits", grid, smem, mx, mw, p, s, "moe_route: logits");
+  // A two-stage ring holds too little to cover an HBM load's way (~1.1 us a k-block), so the x tile
+  // of a stage's next use goes to L2 while this one loads: 78.0 / 72.6 us at T=32768, d=4096,
+  // 128 experts, 62.2 / 56.3 at 64, 428 / 412 at T=65536, d=7168, 208. Not with more stages (no gain
+  // at 28 and 112 experts, 3 stages), nor above 208 experts, where the weights are most of a stage
+  // (277 / 283 at T=65536, d=4096, 240), nor where a tile's rows straddle 128-byte lines (36.6 / 45.9
+  // at T=16545, d=3336, 49 experts; 30.7 / 32.8 at d=3360), nor over few k-blocks. Further ahead is
+  // slower (73.4 us three, 79 eight k-blocks on), and so it is for x^T dZ (40.9 / 47.8 at T=35700,
+  // d=2856, 57 experts).
+  const bool ahead = stages == 2 && NP <= 208 && plan.kb_per_split >= 16 && d % 64 == 0 &&
+                     (reinterpret_cast<uintptr_t>(x) & 127) == 0;
+  const char *what = "moe_route: logits";
+  return ahead ? launch_route_mma<false, 1, true>("route_logits", grid, smem, mx, mw, p, s, what)
+               : launch_route_mma<false, 1, false>("route_logits", grid, smem, mx, mw, p, s, what);
 }
 
 int launch_route(const uint16_t *x, const float *w, const float *b, const uint8_t *mask, int T,

@@ -76,9 +76,11 @@ def test_route_ties_go_to_lower_index():
                                    # d not a multiple of the 64-wide k-block (zero-filled tail),
                                    # few experts (MMA N = 16), one token, the smallest d
                                    (333, 200, 13), (1, 72, 256), (64, 8, 5), (50, 136, 2),
-                                   # three, two and one weight terms per MMA at the edges of each
-                                   # (80 / 81, 128 / 129 experts), many splits, two tiles per CTA
-                                   (40, 4096, 80), (5000, 1000, 81), (20000, 264, 128), (257, 2048, 129)])
+                                   # many splits of few tokens, none of many, two tiles per CTA
+                                   (40, 4096, 80), (5000, 1000, 81), (20000, 264, 128), (257, 2048, 129),
+                                   # x tiles brought to L2 ahead (two-stage ring, 16 and 17 k-blocks):
+                                   # the last one past T, and one per CTA
+                                   (19999, 1024, 171), (19601, 1088, 64)])
 def test_route_logits_fp32(T, d, E):
     inp = case_inputs(T, d, E, 2, 128, seed=5)
     o = oracle_inputs(inp)
