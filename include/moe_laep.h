@@ -98,7 +98,7 @@ int64_t moe_perm_rows_max(int T, int k, int E);
 
 /* Bytes of scratch `ws` every device entry point below may use for a layer of
  * this shape (one buffer serves all calls of a step issued on one stream).
- * Its first 256 bytes hold the weight-gradient GEMMs' tile counter: the
+ * Its first 256 bytes hold the weight-gradient GEMMs' tile counters: the
  * moe_grouped_ffn_* entry points need a ws of at least 256 bytes (16-byte
  * aligned), and two weight-gradient calls whose kernels may overlap on the GPU
  * need separate workspaces. The other calls use disjoint regions after them, so the router

@@ -32,7 +32,7 @@ constexpr size_t kGemmSchedBytes = 256;
 
 // Workspace layout shared by the entry points (disjoint regions, 256-byte aligned).
 struct WsLayout {
-  size_t gemm_sched;    // int32 [1]               grouped GEMM tile counter (offset 0)
+  size_t gemm_sched;    // int32 [2]               tile counters of the weight-gradient GEMMs (offset 0)
   size_t perm_hist;     // int32 [E * nblk]        moe_permute block histograms
   size_t route_dz3;     // bf16  [3, NP, Tp]       moe_route_bwd logit gradient as three bf16 terms
   size_t route_dw_partial; // fp32 [splits, d, NE] moe_route_bwd split-reduction partial sums
