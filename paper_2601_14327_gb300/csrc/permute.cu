@@ -366,7 +366,12 @@ __global__ void transpose_router_kernel(const float *__restrict__ w, int d, int 
   }
 }
 
-// dx[t] = sum_j dx_perm[row(t,j)] + sum_j d_logits[t,j] * w_t[e_j]
+// dx[t] = sum_j dx_perm[row(t,j)] + sum_j d_logits[t,j] * w_t[e_j]. HBM-bound, so what counts is how
+// many warps have their k loads in flight, and that is set by the registers: 58 without the
+// second sum (not ROUTER), 72 with it, 88 with it and several warps per token (SEG, few tokens). One
+// kernel for all, at 88: 1,287 us instead of 1,197 at T=65536, d=7168, top-8, 66 instead of 40 at
+// T=4096, top-2.
+template <bool ROUTER, bool SEG>
 __global__ void __launch_bounds__(kThreads) permute_bwd_kernel(
     const uint16_t *__restrict__ dx_perm, const int32_t *__restrict__ row_of_assignment,
     const int32_t *__restrict__ topk_idx, const float *__restrict__ d_logits,
@@ -374,8 +379,8 @@ __global__ void __launch_bounds__(kThreads) permute_bwd_kernel(
   pdl_start();
   const int lane = threadIdx.x & 31;
   int t, seg;
-  if (!token_segment(blockIdx.x, T, nseg, &t, &seg)) return;
-  const bool router = (d_logits != nullptr && w_t != nullptr);
+  if (!token_segment(blockIdx.x, T, SEG ? nseg : 1, &t, &seg)) return;
+  const bool router = ROUTER && d_logits != nullptr && w_t != nullptr;
   int my_row = (lane < k) ? row_of_assignment[size_t(t) * k + lane] : -1;
   int my_e = (lane < k && router) ? topk_idx[size_t(t) * k + lane] : -1;
   float my_dz = (lane < k && router) ? d_logits[size_t(t) * k + lane] : 0.f;
@@ -388,8 +393,8 @@ __global__ void __launch_bounds__(kThreads) permute_bwd_kernel(
     if (ex[j] >= E) ex[j] = -1;
     dz[j] = __shfl_sync(0xffffffffu, my_dz, j);
   }
-  const int nv = d / 8;
-  for (int c = lane + 32 * seg; c < nv; c += 32 * nseg) {
+  const int nv = d / 8, step = SEG ? 32 * nseg : 32;
+  for (int c = lane + 32 * seg; c < nv; c += step) {
     uint4 v[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j)
@@ -594,7 +599,9 @@ int moe_permute_bwd(const uint16_t *dx_perm, const int32_t *row_of_assignment,
     if (int st = moe::launch_status("moe_permute_bwd: transpose")) return st;
   }
   const int nseg = token_segments(T, d, kCombineWarpsPerSm);
-  MOE_LAUNCH("permute_bwd", s, moe::launch_dep(permute_bwd_kernel, token_grid(T, nseg), kThreads, 0, s, dx_perm,
+  auto kern = d_logits && w_t ? (nseg > 1 ? permute_bwd_kernel<true, true> : permute_bwd_kernel<true, false>)
+                              : (nseg > 1 ? permute_bwd_kernel<false, true> : permute_bwd_kernel<false, false>);
+  MOE_LAUNCH("permute_bwd", s, moe::launch_dep(kern, token_grid(T, nseg), kThreads, 0, s, dx_perm,
                                                row_of_assignment, topk_idx, d_logits, w_t, T, d, E, k, nseg, dx));
   return moe::launch_status("moe_permute_bwd: launch");
 }
