@@ -525,7 +525,8 @@ def test_one_sm_gemm_kernel_against_oracle(one_sm):
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
 
 
-@pytest.mark.parametrize("T,d,E,k,F", [(1500, 384, 12, 4, 640), (3000, 256, 256, 8, 256)])
+@pytest.mark.parametrize("T,d,E,k,F", [(1500, 384, 12, 4, 640), (3000, 256, 256, 8, 256),
+                                       (45, 1152, 9, 3, 256)])  # several warps per token
 def test_router_term_in_dx_epilogue_equals_unpermute_sum_form(T, d, E, k, F):
     """The router's share of dx, added per grouped row in the dX GEMM's epilogue (the
     layer's default), against the same term added per token by moe_permute_bwd: both
