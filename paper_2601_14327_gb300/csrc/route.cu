@@ -68,7 +68,9 @@ int route_tc_np(int E) { return (E + 15) / 16 * 16; }
 // its own, added at the end; the x tile is then read from shared memory once (up to 80 experts)
 // or twice (up to 128) per k-step instead of three times, and shared memory sets the pace of
 // these short-N MMAs: 43 / 31 us at T=16384, d=4096, 64 experts, 47 / 40 us at T=35700, d=2856, 57.
-int route_dw_group(int NP) { return std::min(3, 256 / NP); }
+// At least one: the workspace is also sized for expert counts that moe_route and moe_route_bwd
+// refuse (E > 256), and the plan divides by this.
+int route_dw_group(int NP) { return std::max(1, std::min(3, 256 / NP)); }
 uint32_t route_tc_tmem_cols(int c, int MT) {  // c: accumulator columns of one tile
   if (MT == 2) return 512u;
   return c <= 32 ? 32u : (c <= 64 ? 64u : (c <= 128 ? 128u : 256u));

@@ -4,6 +4,7 @@ validation fails cleanly before any launch."""
 import json
 import os
 import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -43,6 +44,19 @@ def test_sizes(lib):
     assert ws >= 3 * 64 * 16384 * 2 + 4096 * 64 * 4 + 64 * 4096 * 4 + 16384 * 64 * 4 \
         + 3 * 64 * 4096 * 2
     assert L.moe_workspace_size(0, 4096, 64, 8, 2048) >= 64 * 4096 * 4
+
+
+@pytest.mark.parametrize("E", [256, 257, 272, 1000, 100000])
+def test_workspace_size_above_256_experts(lib, E):
+    """moe_workspace_size answers for expert counts that the entry points refuse; in a child
+    process, since an arithmetic trap would end this one."""
+    code = ("from paper_2601_14327_gb300 import _lib as L; "
+            f"print(*[L.moe_workspace_size(T, 4096, {E}, 8, 2048) for T in (0, 1, 1000)])")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=B.ROOT)
+    assert r.returncode == 0, (r.returncode, r.stderr[-500:])
+    s0, s1, s1000 = map(int, r.stdout.split())
+    # the transposed router [E, d] fp32 alone, then per token the dZ terms [3, E] bf16 as well
+    assert E * 4096 * 4 <= s0 < s1 and s1 + 900 * 3 * 2 * E <= s1000
 
 
 def test_laep_prune_mask_golden(lib):
