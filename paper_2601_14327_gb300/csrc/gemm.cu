@@ -121,11 +121,11 @@ struct GemmParams {
   const float *row_dz;
   const float *w_router;
   // kDgradDown with the gate gradient (nullptr: without): for every grouped row r,
-  // gate_partial[r * gate_stride + nt * 2 + half] = sum over the tile's column half of
-  // dH[r, f] * H[r, f], H = silu(A) * B recomputed from the saved pre-activations; the
-  // row's sum over its partials is g * <dy, O> (dH = g * dy W_down).
+  // gate_partial[r * F/64 + i] = sum over columns f = 64 i .. 64 i + 63 of dH[r, f] * H[r, f],
+  // H = silu(A) * B recomputed from the saved pre-activations; the row's sum over its
+  // partials is g * <dy, O> (dH = g * dy W_down). The 64 columns do not depend on the tile's
+  // width, which follows from the rows allocated: neither do the sums' last bits.
   float *gate_partial;
-  int gate_stride;
   // kDgradDown ahead of a dX GEMM with the router's term (nullptr: without): zeroed for every
   // grouped row; the rows of assignments are written between the two GEMMs.
   float *zero_dz;
@@ -245,7 +245,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams &p, const CUtenso
     const int F = p.F;
     const int f0 = nt * BN;
     const int trow = int(row) - lane;
-    float gsum = 0.f;  // this row's sum of dH * H over the warp's columns
+    float gsum = 0.f, gsum0 = 0.f;  // this row's sum of dH * H over 64 columns, and over the 64 before
 #pragma unroll 1
     for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
       if (f0 + c >= F) break;  // a cut last tile
@@ -277,9 +277,17 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams &p, const CUtenso
       }
       stage_and_store(tmO, stage, lane, vda, f0 + c, trow);
       stage_and_store(tmO, stage, lane, vdb, F + f0 + c, trow);
+      if (BN == 256 && c == half * 128 + 32) {
+        gsum0 = gsum;
+        gsum = 0.f;
+      }
+    }
+    if (p.gate_partial != nullptr && f0 + half * (BN / 2) < F) {
+      float *dst = p.gate_partial + row * size_t(F / 64) + (f0 + half * (BN / 2)) / 64;
+      if (BN == 256) *reinterpret_cast<float2 *>(dst) = make_float2(gsum0, gsum);
+      else *dst = gsum;
     }
     if (p.zero_dz != nullptr && nt == 0 && half == 0) p.zero_dz[row] = 0.f;
-    if (p.gate_partial != nullptr) p.gate_partial[row * p.gate_stride + nt * 2 + half] = gsum;
   } else {
     int trow;
     if (Tr::WGRAD) {
@@ -1829,7 +1837,6 @@ int moe_grouped_ffn_bwd_dgrad(const uint16_t *d_out_perm, const uint16_t *ab_sav
   if (!router && !gate && (topk_gate || row_of_assignment))
     return moe::set_error(MOE_ERR_ARG, "%s: routing arguments without a router term or d_gate_out", fn);
   int64_t Rr = 0;
-  int gate_stride = 0;
   moe::WsLayout L{};
   if (router || gate) {
     if (T < 0 || k < 1 || k > 8 || k > E) return moe::set_error(MOE_ERR_ARG, "%s: T=%d k=%d", fn, T, k);
@@ -1848,12 +1855,7 @@ int moe_grouped_ffn_bwd_dgrad(const uint16_t *d_out_perm, const uint16_t *ab_sav
   p.nkb = d / BK;
   p.out = d_ab;
   p.aux = ab_saved;
-  if (gate) {
-    const int cols = act_plan(false, F, d, rows_cap, E).bn;  // the dH GEMM's column tile
-    gate_stride = 2 * ((F + cols - 1) / cols);  // column halves of the N tiles
-    p.gate_partial = reinterpret_cast<float *>(static_cast<char *>(ws) + L.gate_partial);
-    p.gate_stride = gate_stride;
-  }
+  if (gate) p.gate_partial = reinterpret_cast<float *>(static_cast<char *>(ws) + L.gate_partial);
   float *row_dz = router ? reinterpret_cast<float *>(static_cast<char *>(ws) + L.row_dz) : nullptr;
   p.zero_dz = row_dz;
   if ((st = run_gemm<kDgradDown>(F, d_out_perm, R, d, w_down, uint64_t(E) * d, F, R, 2 * F, p,
@@ -1861,7 +1863,7 @@ int moe_grouped_ffn_bwd_dgrad(const uint16_t *d_out_perm, const uint16_t *ab_sav
     return st;
   if (T > 0 && (gate || router)) {
     const float *part = p.gate_partial;
-    const int stride = p.gate_stride, grid = grid_for(int64_t(T) * 8);
+    const int stride = F / 64, grid = grid_for(int64_t(T) * 8);
     if (gate && router)
       MOE_LAUNCH("row_gates", s, moe::launch_dep(row_gates_kernel<true, true>, grid, 256, 0, s, part, stride, topk_gate,
                                                  row_of_assignment, T, k, Rr, d_gate, d_gate_out, row_dz));

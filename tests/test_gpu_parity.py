@@ -593,6 +593,31 @@ def test_gate_gradient_from_dh_epilogue(T, d, E, k, F):
     assert_close("d_logits", b.d_logits.cpu().numpy(), ref["d_logits"])
 
 
+@pytest.mark.parametrize("T,d,E,k,F", [(1021, 512, 32, 4, 512),  # dH tiles 256 and 128 wide
+                                       (1500, 256, 16, 4, 640),  # 128 and 256 wide with a cut last one
+                                       (300, 128, 4, 2, 128)])
+def test_router_gradients_do_not_depend_on_the_rows_allocated(T, d, E, k, F):
+    """More rows allocated than the layout needs can change the dH GEMM's kernel and tile
+    width, but no result: d_gate, the router's logit gradient and dx_perm keep their bits."""
+    b = run_gpu_layer(case_inputs(T, d, E, k, F, seed=T + 5), E, k)
+    g = {n: v.cuda() for n, v in case_inputs(T, d, E, k, F, seed=T + 5).items()}
+    used = int(b.group_offsets[-1])
+    for extra in (4096, 128 * 640 * E):
+        R = b.shape.rows_cap + extra
+        grow = lambda t: torch.cat([t, torch.zeros(R - t.shape[0], t.shape[1], dtype=t.dtype, device="cuda")])
+        d_out, ab = grow(b.d_out_perm), grow(b.ab)
+        d_ab, dx_perm = torch.empty_like(ab), torch.empty_like(d_out)
+        d_gate = torch.full_like(b.d_gate, 7)
+        L.moe_grouped_ffn_bwd_dgrad(d_out, ab, b.group_offsets, E, d, F, R, g["w_gate_up"],
+                                    g["w_down"], b.topk_gate, None, b.row_of_assignment,
+                                    g["w_router"], T, k, d_gate, d_ab, dx_perm, b.ws, b.ws_bytes)
+        torch.cuda.synchronize()
+        assert L.moe_device_error(clear=True) == 0
+        assert torch.equal(d_gate, b.d_gate)
+        assert torch.equal(dx_perm[:used], b.dx_perm[:used])
+        assert torch.equal(d_ab[:used], b.d_ab[:used])
+
+
 def test_dynamic_schedule_equals_fixed_stride(tmp_path):
     """The CTA pairs claim tiles from a shared counter, so which pair computes a tile
     changes from run to run, but not the tile's arithmetic: every output and gradient
