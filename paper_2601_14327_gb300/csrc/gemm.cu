@@ -991,9 +991,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc::tma_gather4_pair(a_dst + uint32_t(lane) * 512u, &tmA, fb, k0, rows4.x, rows4.y,
                                  rows4.z, rows4.w);
           } else if (box < BNH / 64) {
-            tc::tma_gather4_pair(b_dst + uint32_t(box) * 64u * 128u + uint32_t(grp) * 512u, &tmB, fb,
-                                 t.nt * BN + int(rank) * BNH + box * 64, rows4.x, rows4.y, rows4.z,
-                                 rows4.w);
+            // The odd CTA's half of a cut last tile lies past x's last column: it gathers the
+            // even CTA's columns instead (its results are not stored), since a gather, unlike
+            // the tile loads, is only issued inside its tensor here.
+            int col = t.nt * BN + int(rank) * BNH + box * 64;
+            if (col >= p.n_cols) col -= BNH;
+            tc::tma_gather4_pair(b_dst + uint32_t(box) * 64u * 128u + uint32_t(grp) * 512u, &tmB, fb, col,
+                                 rows4.x, rows4.y, rows4.z, rows4.w);
           }
         }
       }

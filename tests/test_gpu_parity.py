@@ -489,7 +489,10 @@ def _layer_both_ways(inp, E, k, mask=None):
                                                 (777, 384, 24, 8, 128, 5),
                                                 (1, 128, 8, 2, 128, 0),
                                                 (0, 128, 4, 2, 128, 0),
-                                                (2048, 256, 8, 1, 384, 3)])
+                                                (2048, 256, 8, 1, 384, 3),
+                                                # dW_gate_up in 256-wide tiles, the last one cut
+                                                (5000, 640, 128, 3, 384, 0),
+                                                (900, 896, 100, 2, 256, 7)])
 def test_gathered_layer_equals_materialized(T, d, E, k, F, n_masked):
     """The gathered dispatch (X_perm never written) gives the materialized path's results
     bit for bit: outputs, every gradient, and the saved activations on real rows."""
