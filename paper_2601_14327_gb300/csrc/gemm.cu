@@ -1386,11 +1386,14 @@ bool split_rows(uint64_t rows) {
 //   then): 128. dH 13.9 / 20.0 us at 1,021 tokens, top-4, 32 experts, d 512, d_ff 384.
 // - Tiles of 256 for at most half the pairs: 128, twice as many pairs work for half as long.
 //   down 8.2 us against 9.1 us at 512 tokens, top-2, 16 experts, d 256, d_ff 512.
-int tile_cols(int N, int64_t row_pairs) {
+// - Gathered columns cost what they take to issue, used or not: a cut tile from N = 896 (a
+//   weight-gradient call 128-wide / cut: 640 / 690 us at N = 384, 102.7 / 104.8 at 640, 48.9 /
+//   47.7 at 896, 396 / 360 at 1408, 336 / 291 at 3200).
+int tile_cols(int N, int64_t row_pairs, bool gather = false) {
   if (N < 256) return 128;
   const int64_t pairs = moe::num_sms() / 2, wide = row_pairs * ((N + 255) / 256);
   if (2 * wide <= pairs) return 128;
-  return N % 256 == 0 || wide >= 3 * pairs ? 256 : 128;
+  return N % 256 == 0 || (wide >= 3 * pairs && !(gather && N < 896)) ? 256 : 128;
 }
 // Row pairs of the activation GEMMs' tile lists, about: every expert's rows in pairs of
 // 128-row blocks, from the rows allocated (T*k + 128 E); half a pair more per expert.
@@ -1443,7 +1446,7 @@ GemmPlan wgrad_plan(int N, int m_tiles, int64_t rows_cap, int E, bool gather) {
   const int forced = forced_one_sm();
   const bool few = A <= int64_t(128) * E || (A <= int64_t(640) * E && tiles <= 2 * moe::num_sms());
   if (!gather && (forced == 1 || (forced < 0 && few))) return {false, N >= 256 ? 256 : 128};
-  return {forced != 1, tile_cols(N, int64_t(E) * ((m_tiles + 1) / 2))};
+  return {forced != 1, tile_cols(N, int64_t(E) * ((m_tiles + 1) / 2), gather)};
 }
 
 // Builds the tensor maps for one GEMM and launches it. A: [a_rows, a_cols] row-major

@@ -490,7 +490,8 @@ def _layer_both_ways(inp, E, k, mask=None):
                                                 (1, 128, 8, 2, 128, 0),
                                                 (0, 128, 4, 2, 128, 0),
                                                 (2048, 256, 8, 1, 384, 3),
-                                                # dW_gate_up in 256-wide tiles, the last one cut
+                                                # dW_gate_up in 128-wide tiles, and in 256-wide
+                                                # ones with a cut last one
                                                 (5000, 640, 128, 3, 384, 0),
                                                 (900, 896, 100, 2, 256, 7)])
 def test_gathered_layer_equals_materialized(T, d, E, k, F, n_masked):
