@@ -107,7 +107,7 @@ def _ptr(t):
     return t.data_ptr()
 
 
-_raw_stream = _cur_device = None
+_current = None  # (handle of a device's current stream, current device), once CUDA is initialized
 
 
 def stream_handle(stream=None) -> int:
@@ -118,14 +118,16 @@ def stream_handle(stream=None) -> int:
     Callers of several entry points read it once and pass it on.
     """
     if stream is None:
-        global _raw_stream, _cur_device
-        if _raw_stream is None:
+        global _current
+        cur = _current
+        if cur is None:
             import torch
             torch.cuda.current_stream()  # initializes CUDA
-            _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream",
-                                  lambda device: torch.cuda.current_stream(device).cuda_stream)
-            _cur_device = torch.cuda.current_device
-        return _raw_stream(_cur_device())
+            # one assignment: another thread sees both functions or neither
+            cur = _current = (getattr(torch._C, "_cuda_getCurrentRawStream",
+                                      lambda device: torch.cuda.current_stream(device).cuda_stream),
+                              torch.cuda.current_device)
+        return cur[0](cur[1]())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -1,10 +1,12 @@
 """C ABI checks that need no GPU: the library builds, loads and exports every
 declared entry point; the host-side LAEP decision matches the oracle; argument
 validation fails cleanly before any launch."""
+import importlib.util
 import json
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -122,6 +124,59 @@ def test_argument_validation_without_launch(lib):
     assert e.value.status == -6
     with pytest.raises(L.MoEError):
         L.laep_prune_mask([1, 2, 3], 2, 4)  # k > E
+
+
+def test_stream_handle_first_calls_from_two_threads(monkeypatch):
+    """The first look-up of the current stream's handle, interrupted at each of its lines by
+    another thread's call: both get their own thread's handle."""
+    import torch
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: None)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream",
+                        lambda dev: (dev, threading.get_ident()), raising=False)
+    spec = importlib.util.spec_from_file_location("paper_2601_14327_gb300._lib_fresh", L.__file__)
+
+    def interrupted_at(n):
+        """Lines of the first look-up that were reached (up to n), and the other call's error."""
+        fresh = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(fresh)
+        lines, failed = 0, []
+
+        def other():
+            try:
+                assert fresh.stream_handle() == (3, threading.get_ident())
+            except Exception as e:
+                failed.append(repr(e))
+
+        def tracer(frame, event, arg):
+            nonlocal lines
+            if frame.f_code.co_filename != fresh.__file__:
+                return None
+            if event == "line" and lines < n:
+                lines += 1
+                if lines == n:
+                    t = threading.Thread(target=other)
+                    t.start()
+                    t.join()
+            return tracer
+
+        old = sys.gettrace()
+        sys.settrace(tracer)
+        try:
+            got = fresh.stream_handle()
+        finally:
+            sys.settrace(old)
+        assert got == (3, threading.get_ident())
+        return lines, failed
+
+    n = 0
+    while True:
+        n += 1
+        lines, failed = interrupted_at(n)
+        assert not failed, (n, failed)
+        if lines < n:
+            break
+    assert n > 3
 
 
 def test_laep_algorithms_golden(lib):
