@@ -28,18 +28,51 @@ __global__ void __launch_bounds__(kRankThreads) perm_hist_kernel(const int32_t *
                                                                  int64_t A, int E,
                                                                  int32_t *__restrict__ hist) {
   __shared__ int sh[256];
-  for (int e = threadIdx.x; e < E; e += kRankThreads) sh[e] = 0;
+  for (int e = threadIdx.x; e < E; e += blockDim.x) sh[e] = 0;
   __syncthreads();
   pdl_start();
   const int64_t a0 = int64_t(blockIdx.x) * kChunk;
   const int64_t a1 = min(A, a0 + kChunk);
-  for (int64_t a = a0 + threadIdx.x; a < a1; a += kRankThreads) {
+  for (int64_t a = a0 + threadIdx.x; a < a1; a += blockDim.x) {
     const int e = idx[a];
     if (e >= 0 && e < E) atomicAdd(&sh[e], 1);
     else dev_flag(&g_dev_err, MOE_DEV_BAD_EXPERT);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < E; e += kRankThreads) hist[size_t(blockIdx.x) * E + e] = sh[e];
+  for (int e = threadIdx.x; e < E; e += blockDim.x) hist[size_t(blockIdx.x) * E + e] = sh[e];
+}
+
+// Many chunks: the block histograms are summed over the chunks once, in place (afterwards
+// hist[b * E + e] counts chunks 0..b), so that a rank block reads two of their rows and not all
+// nblk: that pass is quadratic in the chunks. A block takes 32 experts, one per lane; its warps
+// take kPrefixRows consecutive chunks each, kRankWarps * kPrefixRows per turn.
+constexpr int kPrefixRows = 16;
+__global__ void __launch_bounds__(kRankThreads) perm_prefix_kernel(int32_t *__restrict__ hist, int E, int nblk) {
+  __shared__ int sum[kRankWarps][32];
+  pdl_start();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+  int before = 0;  // of this expert in the chunks of earlier turns
+  for (int b0 = 0; b0 < nblk; b0 += kRankWarps * kPrefixRows) {
+    const int b1 = b0 + warp * kPrefixRows;
+    int v[kPrefixRows];
+#pragma unroll
+    for (int i = 0; i < kPrefixRows; ++i) v[i] = e < E && b1 + i < nblk ? hist[size_t(b1 + i) * E + e] : 0;
+#pragma unroll
+    for (int i = 1; i < kPrefixRows; ++i) v[i] += v[i - 1];
+    sum[warp][lane] = v[kPrefixRows - 1];
+    __syncthreads();
+    int own = before;
+#pragma unroll 8
+    for (int w = 0; w < kRankWarps; ++w) {
+      const int c = sum[w][lane];
+      if (w < warp) own += c;
+      before += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kPrefixRows; ++i)
+      if (e < E && b1 + i < nblk) hist[size_t(b1 + i) * E + e] = own + v[i];
+  }
 }
 
 // Row of every assignment: group start + rank among the earlier assignments of the same
@@ -48,11 +81,15 @@ __global__ void __launch_bounds__(kRankThreads) perm_hist_kernel(const int32_t *
 // - ranks inside the block: warps own consecutive 128-assignment sub-chunks in 32-wide steps;
 //   lanes with equal experts are ranked by lane order, earlier steps by a per-warp count;
 // - the counts of the chunks before it and of all chunks, from the block histograms (one pass
-//   over nblk * E entries from L2 per block; a single chunk needs no histogram kernel);
+//   over nblk * E entries from L2 per block, or their sums over the chunks from
+//   perm_prefix_kernel; a single chunk needs no histogram kernel);
 // - the scan of the padded group sizes (every block, 8 warps).
 // Histogram + scan + rank kernels took 5.7 + 4.5 + 8.4 us and two gaps at T=16384, top-8, 64
 // experts (32 chunks), 2.9 + 2.8 + 7.7 us at T=512, top-2; one kernel takes 5.2 us there now.
-__global__ void __launch_bounds__(kRankThreads) perm_rank_kernel(
+// MANY: hist holds the sums over the chunks, and 32 registers leave room for two blocks per SM
+// (51 without that bound, which the few blocks of a small layout are faster with).
+template <bool MANY>
+__global__ void __launch_bounds__(kRankThreads, MANY ? 2 : 1) perm_rank_kernel(
     const int32_t *__restrict__ idx, int64_t A, int E, int nblk, const int32_t *__restrict__ hist,
     const int32_t *__restrict__ counts_check, int64_t rows_cap, int32_t *__restrict__ group_offsets,
     int32_t *__restrict__ group_counts, int32_t *__restrict__ row_of_assignment, int k,
@@ -61,8 +98,8 @@ __global__ void __launch_bounds__(kRankThreads) perm_rank_kernel(
   __shared__ int part[kRankGroups][2][256];
   __shared__ int s_warp[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < kRankWarps * 256; i += kRankThreads) (&wh[0][0])[i] = 0;
-  __syncthreads();
+  for (int i = lane; i < E; i += 32) wh[warp][i] = 0;  // (only this warp uses it at first)
+  __syncwarp();
   pdl_start();
   const int64_t a0 = int64_t(blockIdx.x) * kChunk + int64_t(warp) * (kRankSteps * 32) + lane;
   int e[kRankSteps], pos[kRankSteps];
@@ -81,7 +118,12 @@ __global__ void __launch_bounds__(kRankThreads) perm_rank_kernel(
   const int ex = tid & 255, grp = tid >> 8;
   if (nblk > 1) {
     int before = 0, all = 0;
-    if (ex < E) {
+    if (MANY) {
+      if (grp == 0 && ex < E) {
+        all = hist[size_t(nblk - 1) * E + ex];
+        before = blockIdx.x > 0 ? hist[size_t(blockIdx.x - 1) * E + ex] : 0;
+      }
+    } else if (ex < E) {
 #pragma unroll 8
       for (int b = grp; b < nblk; b += kRankGroups) {
         const int v = hist[size_t(b) * E + ex];
@@ -106,11 +148,13 @@ __global__ void __launch_bounds__(kRankThreads) perm_rank_kernel(
   // thread ex of the first 256: the expert's counts per warp -> exclusive, its total, its group
   if (tid < 256) {
     int own = 0;
+    if (ex < E) {
 #pragma unroll 8
-    for (int w = 0; w < kRankWarps; ++w) {
-      const int c = wh[w][ex];
-      wh[w][ex] = own;
-      own += c;
+      for (int w = 0; w < kRankWarps; ++w) {
+        const int c = wh[w][ex];
+        wh[w][ex] = own;
+        own += c;
+      }
     }
     int before = 0, cnt = own;
     if (nblk > 1) {
@@ -440,17 +484,28 @@ int token_segments(int T, int d, int per_sm) {
 int token_grid(int T, int nseg) { return int((int64_t(T) * nseg + kWarps - 1) / kWarps); }
 
 // The grouped layout: group_offsets, group_counts, row_of_assignment (and token_of_row when
-// given). One chunk of assignments is one launch; more take the block histograms first.
+// given). One chunk of assignments is one launch; more take the block histograms first, and more
+// than one chunk per SM their sums over the chunks. moe_permute_map, every rank block reading all
+// histograms / with the sums: 16.2 / 21.8 us at 128 chunks of 256 experts, 26.4 / 22.3 at 160,
+// 20.6 / 20.9 at 192 of 64, 70 / 39 at 512 of 256, 541 / 118 at 2,048. (The histogram kernel's
+// blocks: 1,024 threads 38.6 us, 256 threads 39.3 at 512 chunks; 62.5 and 61.1 at 1,024.)
 int launch_layout(const int32_t *idx, int64_t A, int E, int32_t *hist, const int32_t *counts,
                   int64_t rows_cap, int32_t *group_offsets, int32_t *group_counts, int32_t *row, int k,
                   int32_t *token_of_row, cudaStream_t s, const char *what) {
   const int nblk = int(std::max<int64_t>(1, (A + kChunk - 1) / kChunk));
+  const bool many = nblk > moe::num_sms();
   if (nblk > 1) {
-    MOE_LAUNCH("perm_hist", s, moe::launch_dep(perm_hist_kernel, nblk, kRankThreads, 0, s, idx, A, E, hist));
+    const int threads = nblk > 4 * moe::num_sms() ? 256 : kRankThreads;
+    MOE_LAUNCH("perm_hist", s, moe::launch_dep(perm_hist_kernel, nblk, threads, 0, s, idx, A, E, hist));
     if (int st = moe::launch_status(what)) return st;
   }
-  MOE_LAUNCH("perm_rank", s, moe::launch_dep(perm_rank_kernel, nblk, kRankThreads, 0, s, idx, A, E, nblk, hist, counts,
-                                             rows_cap, group_offsets, group_counts, row, k, token_of_row));
+  if (many) {
+    MOE_LAUNCH("perm_prefix", s, moe::launch_dep(perm_prefix_kernel, (E + 31) / 32, kRankThreads, 0, s, hist, E, nblk));
+    if (int st = moe::launch_status(what)) return st;
+  }
+  auto kern = many ? perm_rank_kernel<true> : perm_rank_kernel<false>;
+  MOE_LAUNCH("perm_rank", s, moe::launch_dep(kern, nblk, kRankThreads, 0, s, idx, A, E, nblk, hist, counts, rows_cap,
+                                             group_offsets, group_counts, row, k, token_of_row));
   return moe::launch_status(what);
 }
 

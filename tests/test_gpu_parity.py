@@ -254,6 +254,24 @@ def test_permute_chunk_edges(T, d, E, k):
     assert torch.equal(xp[:int(ooff[-1])], want)
 
 
+@pytest.mark.parametrize("T,E,k", [(77824, 40, 8), (77825, 33, 8),  # 152 chunks, and one more: their
+                                   (262144, 32, 8), (262145, 1, 1),  # histograms summed first
+                                   (262144 + 513, 256, 8), (2100000, 8, 1)])
+def test_permute_many_chunks(T, E, k):
+    """Layout and rows over many chunks, at the edges of the histogram sums' turns (512 chunks)
+    and of their 32-expert blocks."""
+    rng = np.random.default_rng(T + E)
+    first = (E * rng.random(T) ** 2).astype(np.int64)
+    idx = ((first[:, None] + np.arange(k) * (E // k)) % E).astype(np.int32)
+    x = torch.from_numpy(rng.standard_normal((T, 8)).astype(np.float32)).to(torch.bfloat16)
+    goff, gcnt, row, xp = _permute({"x": x}, idx, E, k, counts=np.bincount(idx.reshape(-1), minlength=E))
+    ooff, ocnt, orow = O.permutation(idx, E, 128)
+    assert (goff == ooff).all() and (gcnt == ocnt).all() and (row == orow).all()
+    want = torch.zeros(int(ooff[-1]), 8, dtype=torch.bfloat16)
+    want[torch.from_numpy(orow.reshape(-1)).long()] = x.repeat_interleave(k, dim=0)
+    assert torch.equal(xp[:int(ooff[-1])], want)
+
+
 def test_permute_all_tokens_one_expert_and_empty():
     T, d, E, k = 700, 128, 8, 1
     inp = case_inputs(T, d, E, k, 128, seed=2)
