@@ -272,7 +272,8 @@ int moe_permute_noalloc(const uint16_t *x, const int32_t *topk_idx, const int32_
  * by a second, one-SM launch on the same stream). With few rows per expert (up to
  * 640 on average, fewer for long reductions) those GEMMs run on single SMs, in
  * 128-row tiles; so do the weight gradients up to 128 rows (or short tile lists), each
- * SM taking every 152nd tile of the list. A tile's arithmetic depends neither on which pair or SM runs it nor
+ * SM taking every 152nd tile of the list (tiles of an expert that holds most of the
+ * rows have an SM to themselves, and the others share the rest). A tile's arithmetic depends neither on which pair or SM runs it nor
  * on the tiles' shape: results are bitwise reproducible.
  * Limits: d % 128 == 0, F % 128 == 0, all pointers 16-byte aligned.
  */

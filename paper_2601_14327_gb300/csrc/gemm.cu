@@ -375,6 +375,55 @@ __device__ __forceinline__ void zero_tile_store(const CUtensorMap *tmO, uint32_t
   }
 }
 
+// Weight gradients on single SMs, one warp: how many CTAs (the first ones, to which the list deals
+// its heaviest tiles) take one tile only, the others sharing the rest of the list. A tile of an
+// expert with most of the rows takes longer than many rounds of light and zero tiles; dealt out
+// evenly, its CTA's share of those came on top. dW_down + dW_gate_up, CTA pairs (whose claims
+// level it) / even deal / this: 57 / 64 / 55 us at 3,340 tokens, top-2, 90 experts, d 512, d_ff 384,
+// one expert with 2,688 of 10,496 rows; 175 / 215 / 166 us at 8,120, top-2, 223, d 512, d_ff 768, 7,808 of
+// 17,664; 119 / 138 / 107 us at 3,979, top-1, 112, d 512, d_ff 1408, 3,712 of 4,352; 185 / 228 / 204 us at
+// 9,982, top-2, 161, d 640, d_ff 896, 9,600 of 21,504 (there the one heavy tile is the bound). Below 1,024
+// rows (16 k-blocks) no tile is that heavy, and the ~1 us of this would show.
+__device__ __forceinline__ int ctas_with_one_tile(const int *s_key, const int *s_order, int E, int per_e, int lane) {
+  const int G = gridDim.x;
+  if (per_e >= G || s_key[s_order[0]] < 1024) return 0;
+  // time of a tile of the expert at list position i, in quarters of a k-block's (0.5 us): the
+  // epilogue takes at least three k-blocks' time, the store of a zero tile one and a half
+  auto cost = [&](int i) {
+    const int key = s_key[s_order[i]];
+    return key < 0 ? 0.f : key == 0 ? 6.f : float(max(12, 4 * (key / BK) + 4));
+  };
+  // the first round gives every CTA one tile: all tiles of `full` experts and some of the next's
+  const int full = G / per_e, some = G - full * per_e;
+  float rest = 0.f;  // cost of the tiles after the first round
+  for (int i = lane; i < E; i += 32)
+    if (i >= full) rest += cost(i) * float(i == full ? per_e - some : per_e);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) rest += __shfl_xor_sync(0xffffffffu, rest, off);
+  // With the tiles of the first i experts alone on their CTAs: the time of the heaviest, or that of
+  // the next expert's tile and an even share of the rest
+  const float first = cost(0);
+  float best = 0.95f * (first + rest / float(G));  // an even deal, unless the gain is worth it
+  int best_i = 0;
+  for (int i = 1 + lane; i <= full && i < E && i * per_e < G; i += 32) {
+    const float t = fmaxf(first, cost(i) + rest / float(G - i * per_e));
+    if (t < best) {
+      best = t;
+      best_i = i;
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const float t = __shfl_xor_sync(0xffffffffu, best, off);
+    const int i = __shfl_xor_sync(0xffffffffu, best_i, off);
+    if (t < best || (t == best && i < best_i)) {
+      best = t;
+      best_i = i;
+    }
+  }
+  return best_i * per_e;
+}
+
 template <int MODE, int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -467,6 +516,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   __syncthreads();
   if (warp == 0) warp_prefix_counts(s_prefix, E, lane);
+  if (Tr::WGRAD && warp == 1) {
+    const int alone = ctas_with_one_tile(s_key, s_order, E, p.m_tiles_w * p.n_tiles, lane);
+    if (lane == 0) misc[2] = alone;
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -474,6 +527,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int total = s_prefix[E];
   pdl_launch();  // only now: a dependent must not take the TMEM columns this kernel waits for
 
+  // This CTA's tiles: blockIdx.x and every tile_step-th after it, up to tile_end
+  const int alone = Tr::WGRAD ? misc[2] : 0;
+  const int tile_step = int(gridDim.x) - alone;
+  const int tile_end = int(blockIdx.x) < alone ? min(total, int(blockIdx.x) + 1) : total;
   auto decode = [&](int tile) {
     int lo = 0, hi = E - 1;
     while (lo < hi) {
@@ -500,7 +557,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
+      for (int tile = blockIdx.x; tile < tile_end && ok; tile += tile_step) {
         const Tile t = decode(tile);
         for (int kb = 0; kb < t.nkb; ++kb, ++it) {
           const int s = it % STAGES;
@@ -555,7 +612,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       uint32_t it = 0, tcount = 0;
       bool ok = true, issued = false;
-      for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
+      for (int tile = blockIdx.x; tile < tile_end && ok; tile += tile_step) {
         const Tile t = decode(tile);
         if (t.nkb == 0) continue;
         const uint32_t a = tcount & 1u, aph = (tcount >> 1) & 1u;
@@ -595,7 +652,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t stage = stage_base + uint32_t(warp - 2) * kStageBytes;
     const int r_in_tile = q * 32 + lane;
     uint32_t tcount = 0;
-    for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
+    for (int tile = blockIdx.x; tile < tile_end; tile += tile_step) {
       const Tile t = decode(tile);
       if (Tr::WGRAD && t.nkb == 0) {
         // empty group: its weight gradient is exactly zero
@@ -1437,8 +1494,8 @@ GemmPlan act_plan(bool gate_up, int N, int K, int64_t rows_cap, int E) {
 // average, and up to 640 while the list is at most two tiles per SM. Above, the pairs' fewer
 // operand bytes and their claims (heaviest tile left to the first free pair) win. Measured over
 // 68 GEMMs of the same random layers, against the pair kernel: 0.90 of its time on average
-// (0.47 at best, 16 -> 8 us), 1.16 at worst (24.8 -> 28.9 us, one expert with most rows). On
-// both sides: R = 304, d 6528, d_ff 512: pair 125 us / one-SM 135 us; R = 83, d 1664, d_ff 640:
+// (0.47 at best, 16 -> 8 us), 1.16 at worst (24.8 -> 28.9 us, one expert with most rows, whose
+// tiles shared their SMs with others then: see ctas_with_one_tile). On both sides: R = 304, d 6528, d_ff 512: pair 125 us / one-SM 135 us; R = 83, d 1664, d_ff 640:
 // 47 / 41 us; R = 186, d 384, d_ff 896, 9 experts: 17.6 / 10.1 us.
 GemmPlan wgrad_plan(int N, int m_tiles, int64_t rows_cap, int E, bool gather) {
   const int64_t A = std::max<int64_t>(0, rows_cap - int64_t(128) * E);  // T * k

@@ -716,6 +716,52 @@ def test_pruned_experts_weight_gradients_untouched(T):
         assert_close("dx", to_np(b.dx), ref["dx"])
 
 
+@pytest.mark.parametrize("T,d,E,F,heavy,live", [
+    (1500, 512, 90, 384, 1400, 12),   # one expert's tiles alone on their SMs, zero tiles on the others
+    (3000, 384, 112, 256, 1300, 3),   # two heavy experts
+    (1100, 256, 200, 128, 1024, 200),  # no expert without rows, the fewest rows that count as heavy
+    (896, 256, 200, 128, 896, 1),     # a block fewer; every other expert empty
+    (2000, 2048, 20, 1024, 1900, 6),  # more tiles per expert than SMs
+])
+def test_weight_gradients_of_skewed_layers(T, d, E, F, heavy, live):
+    """Weight gradients with few rows per expert and one expert (or two) that holds most of them:
+    every element against 64 bits, with nothing left of what the buffers held."""
+    rng = np.random.default_rng(T)
+    idx = rng.integers(0, live, size=(T, 1)).astype(np.int32)
+    idx[:heavy] = 0
+    idx[heavy:2 * heavy] = min(1, live - 1)
+    idx[-live:, 0] = np.arange(live)
+    idx = rng.permutation(E).astype(np.int32)[idx]
+    x = torch.from_numpy(rng.standard_normal((T, d)).astype(np.float32)).to(torch.bfloat16)
+    goff, _, row, xp = _permute({"x": x}, idx, E, 1)
+    R, r = xp.shape[0], torch.from_numpy(row.reshape(-1)).long().cuda()
+    g = torch.Generator(device="cuda").manual_seed(T)
+
+    def grouped(n):  # zero on padding rows
+        t = torch.zeros(R, n, dtype=torch.bfloat16, device="cuda")
+        t[r] = torch.randn(T, n, generator=g, device="cuda").to(torch.bfloat16)
+        return t
+
+    xp = torch.zeros(R, d, dtype=torch.bfloat16, device="cuda").index_copy_(0, r, x.cuda())
+    d_out, h, d_ab = grouped(d), grouped(F), grouped(2 * F)
+    dgu = torch.full((E, 2 * F, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ddn = torch.full((E, d, F), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    L.moe_grouped_ffn_bwd_wgrad(d_out, xp, h, d_ab, torch.from_numpy(goff).cuda(), None, E, d, F, R,
+                                dgu, ddn, ws, 256)
+    torch.cuda.synchronize()
+    assert L.moe_device_error(clear=True) == 0
+    for e in range(E):
+        s = slice(int(goff[e]), int(goff[e + 1]))
+        for got, a, b in ((dgu[e], d_ab, xp), (ddn[e], d_out, h)):
+            a, b = a[s].double(), b[s].double()
+            want = a.T @ b
+            # one bf16 rounding (2^-9, and twice that at most), and fp32 sums of n products, which
+            # lose up to 2^-23 of the sum of their sizes per addition (rounded or cut)
+            bound = 2.0 ** -8 * want.abs() + a.shape[0] * 2.0 ** -23 * (a.abs().T @ b.abs())
+            assert ((got.double() - want).abs() <= bound).all(), e
+
+
 def test_bounded_wait_expires_and_reports():
     """A pipeline wait that nothing satisfies (an mbarrier no one arrives on) gives up
     after its limit: the kernel returns, the device error word reads
