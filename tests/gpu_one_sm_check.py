@@ -49,4 +49,5 @@ if __name__ == "__main__":
     check(1500, 384, 12, 4, 640, 3)  # ragged groups, N not a multiple of 256, empty experts
     check(700, 512, 8, 8, 256, 0)    # k = number of experts
     check(3000, 256, 256, 8, 256, 40)  # the maximum expert count
+    check(300, 128, 1, 1, 128, 0)    # weight gradients of one row block (half a pair's tile)
     print("GEMM kernel: ok")

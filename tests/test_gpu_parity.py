@@ -4,6 +4,7 @@ Integer/index results (routing, counts, grouped layout) must be bit-exact
 when both sides route from the same fp32 logits; floating results must meet
 max|gpu - oracle| / max|oracle| <= 2e-2 (bf16 data, fp32 accumulation).
 """
+import json
 import os
 import subprocess
 import sys
@@ -301,7 +302,7 @@ LAYER_CASES = [
     # T, d, E, k, F, bias, n_masked
     (512, 256, 16, 2, 512, "none", 0),        # the tiny workload
     (300, 128, 1, 1, 128, "none", 0),         # one expert, k=1: a dense SwiGLU MLP; N=128 tiles,
-                                              # a weight-gradient pair with one row block
+                                              # weight gradients of one row block
     (1, 256, 4, 2, 256, "zipf", 0),           # a single token
     (1500, 384, 12, 4, 640, "zipf", 3),       # ragged groups, BN=128 paths, empty groups
     (700, 512, 8, 8, 256, "zipf", 0),         # k = number of experts
@@ -643,19 +644,23 @@ def test_router_gradients_do_not_depend_on_the_rows_allocated(T, d, E, k, F):
 def test_dynamic_schedule_equals_fixed_stride(tmp_path):
     """The CTA pairs claim tiles from a shared counter, so which pair computes a tile
     changes from run to run, but not the tile's arithmetic: every output and gradient
-    equals, bit for bit, the fixed-stride schedule (MOE_GEMM_STATIC=1, read once per
-    process, so that half runs in a child process)."""
+    equals, bit for bit, the fixed-stride schedule (MOE_GEMM_STATIC=1), with the CTA-pair
+    kernel in every GEMM (MOE_GEMM_1SM=0); the variables are read once per process, so both
+    halves run in child processes."""
     import gpu_schedule_check as G
-    path = str(tmp_path / "static.pt")
-    env = dict(os.environ, MOE_GEMM_STATIC="1")
     script = os.path.join(os.path.dirname(os.path.abspath(__file__)), "gpu_schedule_check.py")
-    r = subprocess.run([sys.executable, script, path], env=env, capture_output=True, text=True,
-                       timeout=900)
-    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
-    static = torch.load(path)
-    for i, dyn in enumerate(G.run_cases()):
+    got = []
+    for static in ("0", "1"):
+        path = str(tmp_path / f"{static}.json")
+        env = dict(os.environ, MOE_GEMM_STATIC=static, MOE_GEMM_1SM="0")
+        r = subprocess.run([sys.executable, script, path], env=env, capture_output=True, text=True,
+                           timeout=900)
+        assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+        with open(path) as f:
+            got.append(json.load(f))
+    for case, dyn, static in zip(G.SCHEDULE_CASES, *got):
         for n in G.NAMES:
-            assert torch.equal(dyn[n], static[i][n]), (G.SCHEDULE_CASES[i], n)
+            assert dyn[n] == static[n], (case, n)
 
 
 def test_row_block_split_equals_single_launch(tmp_path):
