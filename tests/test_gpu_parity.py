@@ -936,36 +936,48 @@ def test_fused_combine_without_tokens():
 
 
 def test_back_to_back_steps_equal_synchronised_ones():
-    """Kernels start while their predecessors end (programmatic dependent launches): layer
-    steps of two shapes issued in turn with nothing waiting between, on one workspace each,
-    give the bits that each gives alone."""
-    names = ["y", "dx", "dw_gate_up", "dw_down", "dw_router", "topk_idx", "row_of_assignment",
-             "group_offsets", "d_logits", "counts"]
+    """Kernels start while their predecessors end (programmatic dependent launches): steps on
+    two inputs in turn through ONE set of buffers and one workspace, with nothing waiting between,
+    give the bits that each gives in buffers of its own. Every tensor in between holds the other
+    input's values when a step begins, so a kernel that read one before its predecessor had
+    written it would give other bits; each step's results are copied out on the same stream."""
+    names = ["y", "dx", "dw_gate_up", "dw_down", "dw_router", "topk_idx", "topk_gate",
+             "row_of_assignment", "group_offsets", "d_logits", "d_gate", "counts"]
 
-    def state(T, d, E, k, F, seed):
-        inp = {n: v.cuda() for n, v in case_inputs(T, d, E, k, F, seed=seed).items()}
-        return layer.MoELayerBuffers(layer.LayerShape(T, d, E, k, F), "cuda"), inp
-
-    def step(s):
-        b, g = s
+    def step(b, g):
         layer.forward(b, g["x"], g["w_router"], g["bias"], g["w_gate_up"], g["w_down"])
         layer.backward(b, g["dy"], g["w_router"], g["w_gate_up"], g["w_down"])
 
-    states = [state(777, 256, 16, 4, 384, 1), state(5000, 384, 40, 3, 256, 2)]
-    want = []
-    for s in states:
-        step(s)
+    for T, d, E, k, F in [(777, 256, 16, 4, 384), (5000, 384, 40, 3, 256)]:
+        # other tokens and another bias: another routing, other group offsets
+        inputs = [{n: v.cuda() for n, v in case_inputs(T, d, E, k, F, seed=seed).items()} for seed in (1, 2)]
+        want = []
+        for g in inputs:
+            b = layer.MoELayerBuffers(layer.LayerShape(T, d, E, k, F), "cuda")
+            step(b, g)
+            torch.cuda.synchronize()
+            want.append({n: getattr(b, n).clone() for n in names})
+        for n in ("group_offsets", "y", "d_gate"):
+            assert not torch.equal(want[0][n], want[1][n]), n
+        b = layer.MoELayerBuffers(layer.LayerShape(T, d, E, k, F), "cuda")
+        got = [[{n: torch.empty_like(v) for n, v in w.items()} for w in want] for _ in range(10)]
         torch.cuda.synchronize()
-        want.append({n: getattr(s[0], n).clone() for n in names})
-    for s in states:
+        for turn in got:
+            for i in range(2):
+                step(b, inputs[i])
+                for n, v in turn[i].items():
+                    v.copy_(getattr(b, n))
+        torch.cuda.synchronize()
+        assert L.moe_device_error(clear=True) == 0
+        for turn in got:
+            for i in range(2):
+                for n in names:
+                    assert torch.equal(turn[i][n], want[i][n]), (T, i, n)
+        for i in range(21):  # and with nothing of another kind between the steps
+            step(b, inputs[i % 2])
+        torch.cuda.synchronize()
         for n in names:
-            getattr(s[0], n).fill_(7)
-    for i in range(20):
-        step(states[i % 2])
-    torch.cuda.synchronize()
-    for s, w in zip(states, want):
-        for n in names:
-            assert torch.equal(getattr(s[0], n), w[n]), n
+            assert torch.equal(getattr(b, n), want[0][n]), (T, n)
 
 
 def test_graph_replay_of_the_step_equals_eager():
