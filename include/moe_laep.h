@@ -269,12 +269,13 @@ int moe_permute_noalloc(const uint16_t *x, const int32_t *topk_idx, const int32_
  * of 1-7 k-blocks of 128 rows are claimed 8, 4 or 2 at a time); the other GEMMs'
  * tiles all cost the same, are listed in expert order and each pair takes every
  * 76th one (with rows_cap >= 2^18, a group's odd last 128-row block is computed
- * by a second, one-SM launch on the same stream). With few rows per expert (up to
- * 640 on average, fewer for long reductions) those GEMMs run on single SMs, in
- * 128-row tiles; so do the weight gradients up to 128 rows (or short tile lists), each
- * SM taking every 152nd tile of the list (tiles of an expert that holds most of the
- * rows have an SM to themselves, and the others share the rest). A tile's arithmetic depends neither on which pair or SM runs it nor
- * on the tiles' shape: results are bitwise reproducible.
+ * by a second, one-SM launch on the same stream). With few rows per expert (up to 640
+ * on average over rows_cap - 128 E rows, fewer for long reductions) those GEMMs run on
+ * single SMs, in 128-row tiles; so do the weight gradients up to 128 rows (or short tile
+ * lists), each SM taking every 152nd tile of the list (tiles of an expert that holds most
+ * of the rows have an SM to themselves, and the others share the rest). A tile's arithmetic
+ * depends neither on which pair or SM runs it nor on the tiles' shape, which follows from
+ * rows_cap: results are bitwise reproducible, whatever rows_cap is.
  * Limits: d % 128 == 0, F % 128 == 0, all pointers 16-byte aligned.
  */
 int moe_grouped_ffn_fwd(const uint16_t *x_perm, const int32_t *group_offsets, int E, int d,

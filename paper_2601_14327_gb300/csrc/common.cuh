@@ -82,11 +82,11 @@ namespace moe {
 // Launches a kernel as a programmatic dependent of the one before it on the stream: its
 // blocks may become resident, and run up to their pdl_wait(), while that kernel's last
 // blocks finish. EVERY kernel launched this way calls pdl_wait() in all its threads before it
-// touches memory, so stream order holds for every access, across any number of launches.
+// touches global memory, so stream order holds for every access, across any number of launches.
 // Without it a kernel started ~2 us after its predecessor's end (launch latency and drain),
 // and a layer is a dozen or two launches: with it and fewer launches a forward at T=512,
-// d=256, 16 experts takes 48 us instead of 69, a training step at T=1,021, d=512 140 instead of
-// 209.
+// d=256, 16 experts went from 69 to 48 us (32 us with what came later), a training step at T=1,021,
+// d=512 from 209 to 140 (124).
 template <typename... P, typename... A>
 void launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchAttribute at;

@@ -1312,7 +1312,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 using moe::make_map;
 
 // MOE_GEMM_1SM=1 selects the one-SM kernel and =0 the CTA-pair kernel for every GEMM, whatever
-// the shape (tests and A/B measurements of the two forms); -1: gemm_plan decides.
+// the shape (tests and A/B measurements of the two forms); -1: act_plan and wgrad_plan decide.
 int forced_one_sm() {
   static int v = -2;
   if (v == -2) {
@@ -1435,8 +1435,8 @@ bool split_rows(uint64_t rows) {
 // second half lies past the matrix: its operand boxes are zero-filled without memory reads and
 // it is not stored.
 // - Enough tiles: 256. A CTA of a 256-wide pair tile loads 64 KB per 128-deep k-block where a
-//   128-wide one loads 48 KB for half the columns, and at ~45 B per clock and SM those loads set
-//   the pace. 128-wide / 256-wide with a cut last tile: dH 140 / 122 us and dW_down 112 / 104 us
+//   128-wide one loads 48 KB for half the columns, and at 45-53 B per clock and SM those loads
+//   set the pace. 128-wide / 256-wide with a cut last tile: dH 140 / 122 us and dW_down 112 / 104 us
 //   at 2,039 tokens, top-6, 64 experts, d 2048, d_ff 1408; dX 1951 / 1593 us and dW_gate_up
 //   1970 / 1650 us at 65,396 tokens, top-6, 85 experts, d 2176, d_ff 768.
 // - A cut tile pays its unused half, so below three waves of tiles (the last wave weighs more
@@ -1463,7 +1463,8 @@ int64_t act_row_pairs(int64_t rows_cap, int E) {
 // an expert with up to 128 rows leaves half of each tile unused, and a short list fills its
 // waves badly. The one-SM kernel has twice as many tiles of 128 rows to spread, at ~1.2 times
 // the time per k-block (96 KB of loads per CTA against 64 KB). With R = rows per expert on
-// average, one-SM up to R = 640 and R * K = 3 * 2^18 (a long reduction makes the loads weigh
+// average, taken from the rows allocated (the host does not know the loads; a layer with many more
+// rows allocated than it needs gets the large layers' kernel, and the same results), one-SM up to R = 640 and R * K = 3 * 2^18 (a long reduction makes the loads weigh
 // more than the tile counts). Measured over 134 GEMMs of 34 random layers (R 0.2-1,500, K
 // 256-7168, N 256-7168), against the pair kernel: 0.87 of its time on average, 0.53 at best
 // (10 us class), 1.08 at worst (12.4 -> 13.4 us). On both sides of the line: pair 121 us / one-SM
