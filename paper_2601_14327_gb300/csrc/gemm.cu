@@ -383,44 +383,37 @@ __device__ __forceinline__ void zero_tile_store(const CUtensorMap *tmO, uint32_t
 // one expert with 2,688 of 10,496 rows; 175 / 215 / 166 us at 8,120, top-2, 223, d 512, d_ff 768, 7,808 of
 // 17,664; 119 / 138 / 107 us at 3,979, top-1, 112, d 512, d_ff 1408, 3,712 of 4,352; 185 / 228 / 204 us at
 // 9,982, top-2, 161, d 640, d_ff 896, 9,600 of 21,504 (there the one heavy tile is the bound). Below 1,024
-// rows (16 k-blocks) no tile is that heavy, and the ~1 us of this would show.
+// rows (16 k-blocks) no tile is that heavy, and the time of this (~0.3 us) would show.
 __device__ __forceinline__ int ctas_with_one_tile(const int *s_key, const int *s_order, int E, int per_e, int lane) {
   const int G = gridDim.x;
   if (per_e >= G || s_key[s_order[0]] < 1024) return 0;
   // time of a tile of the expert at list position i, in quarters of a k-block's (0.5 us): the
   // epilogue takes at least three k-blocks' time, the store of a zero tile one and a half
-  auto cost = [&](int i) {
+  auto cost = [&](int i) -> unsigned {
     const int key = s_key[s_order[i]];
-    return key < 0 ? 0.f : key == 0 ? 6.f : float(max(12, 4 * (key / BK) + 4));
+    return key < 0 ? 0u : key == 0 ? 6u : unsigned(max(12, 4 * (key / BK) + 4));
   };
   // the first round gives every CTA one tile: all tiles of `full` experts and some of the next's
   const int full = G / per_e, some = G - full * per_e;
-  float rest = 0.f;  // cost of the tiles after the first round
-  for (int i = lane; i < E; i += 32)
-    if (i >= full) rest += cost(i) * float(i == full ? per_e - some : per_e);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) rest += __shfl_xor_sync(0xffffffffu, rest, off);
+  unsigned after = 0;  // cost of a tile of each expert after those
+  for (int i = full + 1 + lane; i < E; i += 32) after += cost(i);
+  after = __reduce_add_sync(0xffffffffu, after);
+  const float rest = float(after) * float(per_e) + (full < E ? float(cost(full)) * float(per_e - some) : 0.f);
   // With the tiles of the first i experts alone on their CTAs: the time of the heaviest, or that of
   // the next expert's tile and an even share of the rest
-  const float first = cost(0);
+  const float first = float(cost(0));
   float best = 0.95f * (first + rest / float(G));  // an even deal, unless the gain is worth it
   int best_i = 0;
   for (int i = 1 + lane; i <= full && i < E && i * per_e < G; i += 32) {
-    const float t = fmaxf(first, cost(i) + rest / float(G - i * per_e));
+    const float t = fmaxf(first, float(cost(i)) + rest / float(G - i * per_e));
     if (t < best) {
       best = t;
       best_i = i;
     }
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float t = __shfl_xor_sync(0xffffffffu, best, off);
-    const int i = __shfl_xor_sync(0xffffffffu, best_i, off);
-    if (t < best || (t == best && i < best_i)) {
-      best = t;
-      best_i = i;
-    }
-  }
+  // (positive floats order like their bits)
+  const unsigned least = __reduce_min_sync(0xffffffffu, __float_as_uint(best));
+  best_i = int(__reduce_min_sync(0xffffffffu, __float_as_uint(best) == least ? unsigned(best_i) : ~0u));
   return best_i * per_e;
 }
 
