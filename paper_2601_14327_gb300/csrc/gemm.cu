@@ -1667,12 +1667,23 @@ __global__ void row_gates_kernel(const float *__restrict__ partial, int stride,
       if (GATE) {
         if (ok) {
           float s = 0.f;
-          const float2 *src = reinterpret_cast<const float2 *>(partial + size_t(r) * stride);
+          const float *src = partial + size_t(r) * stride;  // (stride = F / 64 is even)
+          if (stride % 4 == 0) {
 #pragma unroll 4
-          for (int c = 0; c < stride / 2; ++c) {
-            const float2 v = src[c];
-            s += v.x;
-            s += v.y;
+            for (int c = 0; c < stride; c += 4) {
+              const float4 v = *reinterpret_cast<const float4 *>(src + c);
+              s += v.x;
+              s += v.y;
+              s += v.z;
+              s += v.w;
+            }
+          } else {
+#pragma unroll 4
+            for (int c = 0; c < stride; c += 2) {
+              const float2 v = *reinterpret_cast<const float2 *>(src + c);
+              s += v.x;
+              s += v.y;
+            }
           }
           dg = g > 0.f ? s / g : 0.f;
           d_gate_out[a] = dg;
