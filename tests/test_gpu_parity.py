@@ -361,8 +361,7 @@ def test_layer_fwd_bwd_against_oracle(T, d, E, k, F, bias, n_masked):
     # CTA pairs (900 rows per expert), >= 3 waves of 256-wide tiles with a cut last one in
     # every GEMM whose N is 384 or 640
     (9000, 384, 40, 4, 640, "zipf", 5),
-    # one-SM activation GEMMs, cut 256-wide tiles, one-block groups and empty experts; CTA-pair
-    # weight gradients with cut tiles
+    # every GEMM on single SMs, cut 256-wide tiles, one-block groups and empty experts
     (5000, 640, 128, 3, 384, "loguniform", 0),
     # one wave either way: 128-wide tiles, N a multiple of 256
     (200, 256, 3, 2, 512, "none", 0),
